@@ -168,6 +168,7 @@ struct vafr_session {
     int2* d_rep_holes = nullptr;
     unsigned* d_rep_count = nullptr;
     void* disp_internal = nullptr;     // render_frame's device display for host output
+    void* d_path = nullptr;            // path tracing scratch (first use)
     int recon_variant = 0;
     int render_variant = 0;
     LptState* d_lpt[2] = {nullptr, nullptr};   // longest-first order state per eye
@@ -188,6 +189,7 @@ struct vafr_session {
         cudaFree(d_rep_holes);
         cudaFree(d_rep_count);
         cudaFree(disp_internal);
+        cudaFree(d_path);
     }
 };
 
@@ -799,7 +801,8 @@ int vafr_render_lp_pt(const vafr_scene* scene, vafr_session* s, int32_t eye_mask
         b.total_work += s->n_texels;
         b.d[b.n++] = f;
     }
-    CUDA_TRY(launch_path_lp(scene->dev, b, (unsigned long long)seed, max_diffuse, as_stream(stream), s->sms));
+    if (!s->d_path) CUDA_TRY(cudaMalloc(&s->d_path, path_scratch_bytes(s->sms)));
+    CUDA_TRY(launch_path_lp(scene->dev, b, (unsigned long long)seed, max_diffuse, s->d_path, as_stream(stream), s->sms));
     return VAFR_OK;
 }
 
@@ -1040,7 +1043,8 @@ int vafr_render_full_gt_pt(const vafr_scene* scene, vafr_session* s, int32_t eye
     b.d[0] = f;
     b.n = 1;
     b.total_work = gt_items(f);
-    CUDA_TRY(launch_path_gt(scene->dev, b, (unsigned long long)seed, max_diffuse, as_stream(stream), s->sms));
+    if (!s->d_path) CUDA_TRY(cudaMalloc(&s->d_path, path_scratch_bytes(s->sms)));
+    CUDA_TRY(launch_path_gt(scene->dev, b, (unsigned long long)seed, max_diffuse, s->d_path, as_stream(stream), s->sms));
     return VAFR_OK;
 }
 

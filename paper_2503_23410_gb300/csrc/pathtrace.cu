@@ -53,184 +53,288 @@ __device__ __forceinline__ float3 face_normal(const SceneDev& sc, const Ray& r, 
     return make_float3(nx, ny, nz);
 }
 
-// One path from the primary ray r; returns the radiance, fills sig (depth + 2
-// ints: hit id per segment, -1 miss, -2 not traced; then the shadow mask: bit k
-// = segment k's shadow ray reached the light, bit 16 + k = it was cast).
-template <int ORDER>
-__device__ float3 trace_path(const SceneDev& sc, Ray r, unsigned long long seed_h, unsigned long long texel,
-                             int depth, int* sig, unsigned* fault) {
-    float3 beta = make_float3(1.0f, 1.0f, 1.0f), acc = make_float3(0.0f, 0.0f, 0.0f);
+// A warp keeps a pool of paths, one record per path that still has a ray to
+// trace: a closest-hit segment or a shadow ray.  It traces 32 records at a
+// time, whatever their depth and kind, and returns the paths that go on to the
+// pool; whenever fewer than 32 are left it starts the next 32 paths.  So every
+// traversal has 32 rays until the work runs out, and the primary rays of a
+// chunk are still traced together.
+//
+// One path per lane from its first to its last segment left most lanes idle:
+// on the 1.07 M triangle terrain 93 % of the paths have a second segment but
+// 25 % a third and 16 % a fourth, and 14 %, 12 % and 7 % a shadow ray there,
+// while each of these steps took a warp as long as the full ones (308, 695,
+// 1,077 and 1,391 us for the LP buffer at 0 to 3 bounces, 10.6 of 32 lanes
+// active).  With the pool: 298, 638, 889 and 1,064 us (15 lanes; the incoherent
+// bounce rays' leaf tests and pushes are what diverges now).
+// The records also hold what the traversal does not need, so it fits 64
+// registers and kPathBlocks blocks per SM (one path per lane: 93 and 5; 6, 7
+// and 8 blocks measured 1,156, 1,148 and 1,110 us, and 1,064 with all four
+// children sorted).  What a ray does not need lies in global memory instead
+// of beside it in shared memory, where it took L1 from the nodes (1,172 us).
+constexpr int kPathBlocks = 8;   // resident blocks per SM that the launch and its scratch count on
+constexpr int kPoolPaths = 64;   // fewer than 32 waiting, and the next 32
+struct PathPool {
+    float o[3][kPoolPaths], d[3][kPoolPaths];   // next ray's origin; direction of the next closest-hit segment
+    int skip[kPoolPaths];                       // triangle the ray leaves
+    unsigned work[kPoolPaths];                  // work item (texel or pixel)
+    unsigned step[kPoolPaths];                  // 2 x segment, + 1: its shadow ray
+};
+// The rest of a record, in global memory (L2): read and written once per ray,
+// and not before a path's first hit (until then beta is 1, the rest 0).
+struct PathState {
+    float beta[3][kPoolPaths], acc[3][kPoolPaths];
+    float cosl[kPoolPaths];      // shadow ray: cosine towards the light
+    unsigned mask[kPoolPaths];   // signature: shadow rays lit / cast
+};
+
+// LP texel or display pixel of a work item: its primary ray and random-number
+// key; false when the item is outside the display.
+template <bool GT>
+__device__ __forceinline__ bool path_ray(const FrameDesc& f, long long local, Ray& r, unsigned long long& key,
+                                         int& slot, int& glo, int& ghi, long long& px) {
+    glo = ghi = -1;
+    if (!GT) {
+        slot = lp_ray(f, (int)local, r, glo, ghi);
+        key = (unsigned long long)(slot - (2 * __ldg(f.work + local).y + 1));   // index in column order, no guards
+        return true;
+    }
+    const long long tile = local >> 5;
+    const int in = (int)(local & 31);
+    const int tiles_x = (f.W + 7) >> 3;
+    const int x = (int)(tile % tiles_x) * 8 + (in & 7);
+    const int y = (int)(tile / tiles_x) * 4 + (in >> 3);
+    if (x >= f.W || y >= f.H) return false;
+    world_ray(f, f.cr * ((float)x + 0.5f - 0.5f * (float)f.W), f.cr * (0.5f * (float)f.H - ((float)y + 0.5f)), r);
+    px = (long long)y * f.W + x;
+    key = (unsigned long long)px;
+    return true;
+}
+
+// Path signature (LP only): depth + 2 ints per slot: hit id per segment, -1
+// miss, -2 not traced; then the shadow mask: bit k = segment k's shadow ray
+// reached the light, bit 16 + k = it was cast.
+template <int TPB, int ORDER, bool GT, int MINB, class B>
+__global__ void __launch_bounds__(TPB, MINB)
+k_path(const SceneDev sc, const __grid_constant__ B b, unsigned long long seed, int depth, PathState* states) {
+    __shared__ PathPool pools[TPB / 32];
+    PathPool& P = pools[threadIdx.x >> 5];
+    PathState& S = states[blockIdx.x * (TPB / 32) + (threadIdx.x >> 5)];
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const unsigned long long seed_h = sm64_mix(seed);
     const float tlx = -sc.light[0], tly = -sc.light[1], tlz = -sc.light[2];
-    unsigned mask = 0u;
-    int k = 0;
-    for (; k <= depth; ++k) {
-        ray_setup(r);
-        Hit h;
-        *fault |= traverse4<false, ORDER, false, true>(sc, r, h, nullptr, nullptr, nullptr);
-        if (sig) sig[k] = h.leaf >= 0 ? h.id : -1;
-        if (h.leaf < 0) {
-            const float3 sky = sky_rgb(r.dx, r.dy, r.dz);
-            acc.x = fmaf(beta.x, sky.x, acc.x);
-            acc.y = fmaf(beta.y, sky.y, acc.y);
-            acc.z = fmaf(beta.z, sky.z, acc.z);
-            ++k;
-            break;
+    int count = 0;          // records in the pool
+    bool more = true;       // work items left
+    while (true) {
+        if (count < 32 && more) {   // the next 32 paths
+            unsigned long long base = 0ull;
+            if (lane == 0) base = atomicAdd(b.work_counter, 32ull);
+            base = __shfl_sync(full, base, 0);
+            more = (long long)base < b.total_work;
+            const long long w = (long long)base + lane;
+            Ray r;
+            unsigned long long key;
+            int slot, glo, ghi;
+            long long px;
+            bool live = w < b.total_work;
+            if (live) {
+                const FrameDesc& f = b.d[find_frame(b, w, false)];
+                live = path_ray<GT>(f, w - f.work_begin, r, key, slot, glo, ghi, px);
+            }
+            const unsigned lm = __ballot_sync(full, live);
+            if (live) {
+                const int q = count + __popc(lm & ((1u << lane) - 1u));
+                P.o[0][q] = r.ox; P.o[1][q] = r.oy; P.o[2][q] = r.oz;
+                P.d[0][q] = r.dx; P.d[1][q] = r.dy; P.d[2][q] = r.dz;
+                P.skip[q] = -1;
+                P.work[q] = (unsigned)w;
+                P.step[q] = 0u;
+            }
+            count += __popc(lm);
+            __syncwarp();
+            if (count < 32 && more) continue;
         }
-        const float3 n = face_normal(sc, r, h.leaf);
-        float px = fmaf(h.t, r.dx, r.ox), py = fmaf(h.t, r.dy, r.oy), pz = fmaf(h.t, r.dz, r.oz);
-        const float off = 1e-5f * fmaxf(1.0f, fmaxf(fabsf(px), fmaxf(fabsf(py), fabsf(pz))));
-        px = fmaf(off, n.x, px);
-        py = fmaf(off, n.y, py);
-        pz = fmaf(off, n.z, pz);
-        const float4 rho = __ldg(sc.albedo + h.id);
-        const float cosl = fmaf(n.x, tlx, fmaf(n.y, tly, n.z * tlz));
-        if (cosl > 0.0f) {
-            mask |= 1u << (16 + k);   // a shadow ray was cast
-            Ray s;
-            s.ox = px; s.oy = py; s.oz = pz;
-            s.dx = tlx; s.dy = tly; s.dz = tlz;
-            s.skip = h.id;
-            ray_setup(s);
-            Hit hs;
-            *fault |= traverse4<false, ORDER, true, true>(sc, s, hs, nullptr, nullptr, nullptr);
-            if (hs.leaf < 0) {
-                mask |= 1u << k;
-                acc.x = fmaf(beta.x * rho.x, cosl, acc.x);
-                acc.y = fmaf(beta.y * rho.y, cosl, acc.y);
-                acc.z = fmaf(beta.z * rho.z, cosl, acc.z);
+        if (count == 0) break;
+        const int n = min(count, 32);
+        const int q = count - n + lane;   // this lane's record
+        const bool on = lane < n;
+        Hit h;
+        if (on) {
+            const bool shadow = P.step[q] & 1u;
+            Ray r;
+            r.ox = P.o[0][q]; r.oy = P.o[1][q]; r.oz = P.o[2][q];
+            r.dx = shadow ? tlx : P.d[0][q];
+            r.dy = shadow ? tly : P.d[1][q];
+            r.dz = shadow ? tlz : P.d[2][q];
+            r.skip = P.skip[q];
+            ray_setup(r);
+            const unsigned fault = traverse4<false, ORDER, true>(sc, r, h, nullptr, nullptr, nullptr, shadow);
+            if (fault) atomicOr(b.d[find_frame(b, (long long)P.work[q], false)].status, fault);
+        }
+        __syncwarp();
+        bool go = false;   // the path has another ray
+        float o[3], d[3], beta[3] = {1.0f, 1.0f, 1.0f}, acc[3] = {0.0f, 0.0f, 0.0f}, cosl = 0.0f;
+        int skip = -1;
+        unsigned work = 0u, step = 0u, mask = 0u;
+        if (on) {
+            work = P.work[q];
+            step = P.step[q];
+            skip = P.skip[q];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                o[c] = P.o[c][q];
+                d[c] = P.d[c][q];
+            }
+            if (step) {
+                mask = __ldcg(&S.mask[q]);
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    beta[c] = __ldcg(&S.beta[c][q]);
+                    acc[c] = __ldcg(&S.acc[c][q]);
+                }
+            }
+            const int k = (int)(step >> 1);
+            const FrameDesc& f = b.d[find_frame(b, (long long)work, false)];
+            const long long local = (long long)work - f.work_begin;
+            Ray r;
+            unsigned long long key = 0ull;
+            int slot = 0, glo = -1, ghi = -1;
+            long long px = 0;
+            path_ray<GT>(f, local, r, key, slot, glo, ghi, px);
+            int* sig = !GT && f.hit_ids ? f.hit_ids + (long long)slot * (depth + 2) : nullptr;
+            if (step & 1u) {
+                if (h.leaf < 0) {
+                    cosl = __ldcg(&S.cosl[q]);
+                    mask |= 1u << k;
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) acc[c] = fmaf(beta[c], cosl, acc[c]);
+                }
+                go = k < depth;
+                step = 2u * (unsigned)(k + 1);
+            } else {
+                if (sig) sig[k] = h.leaf >= 0 ? h.id : -1;
+                if (h.leaf < 0) {
+                    const float3 sky = sky_rgb(d[0], d[1], d[2]);
+                    acc[0] = fmaf(beta[0], sky.x, acc[0]);
+                    acc[1] = fmaf(beta[1], sky.y, acc[1]);
+                    acc[2] = fmaf(beta[2], sky.z, acc[2]);
+                } else {
+                    r.ox = o[0]; r.oy = o[1]; r.oz = o[2];
+                    r.dx = d[0]; r.dy = d[1]; r.dz = d[2];
+                    const float3 nn = face_normal(sc, r, h.leaf);
+                    float pnx = fmaf(h.t, r.dx, r.ox), pny = fmaf(h.t, r.dy, r.oy), pnz = fmaf(h.t, r.dz, r.oz);
+                    const float off = 1e-5f * fmaxf(1.0f, fmaxf(fabsf(pnx), fmaxf(fabsf(pny), fabsf(pnz))));
+                    o[0] = fmaf(off, nn.x, pnx);
+                    o[1] = fmaf(off, nn.y, pny);
+                    o[2] = fmaf(off, nn.z, pnz);
+                    const float4 rho = __ldg(sc.albedo + h.id);
+                    beta[0] *= rho.x; beta[1] *= rho.y; beta[2] *= rho.z;
+                    skip = h.id;
+                    cosl = fmaf(nn.x, tlx, fmaf(nn.y, tly, nn.z * tlz));
+                    if (k < depth) {
+                        const float u1 = pt_uniform(seed_h, key, k, 0), u2 = pt_uniform(seed_h, key, k, 1);
+                        float sp, cp;
+                        sincospif(2.0f * u2, &sp, &cp);
+                        const float rr = sqrtf(u1);
+                        const float lx = rr * cp, ly = rr * sp, lz = sqrtf(fmaxf(0.0f, 1.0f - u1));
+                        const float sg = copysignf(1.0f, nn.z);
+                        const float aa = -1.0f / (sg + nn.z);
+                        const float bb = nn.x * nn.y * aa;
+                        const float t1x = 1.0f + sg * nn.x * nn.x * aa, t1y = sg * bb, t1z = -sg * nn.x;
+                        const float t2x = bb, t2y = sg + nn.y * nn.y * aa, t2z = -nn.y;
+                        d[0] = fmaf(lx, t1x, fmaf(ly, t2x, lz * nn.x));
+                        d[1] = fmaf(lx, t1y, fmaf(ly, t2y, lz * nn.y));
+                        d[2] = fmaf(lx, t1z, fmaf(ly, t2z, lz * nn.z));
+                    }
+                    if (cosl > 0.0f) {   // a shadow ray is cast
+                        mask |= 1u << (16 + k);
+                        step += 1u;
+                        go = true;
+                    } else {
+                        step += 2u;
+                        go = k < depth;
+                    }
+                }
+            }
+            if (!go) {
+                const float4 v = make_float4(acc[0], acc[1], acc[2], 1.0f);
+                if (GT) {
+                    store_px(f.disp, px, f.disp_fmt, v);
+                } else {
+                    store_px(f.lp, slot, f.lp_fmt, v);
+                    if (glo >= 0) store_px(f.lp, glo, f.lp_fmt, v);
+                    if (ghi >= 0) store_px(f.lp, ghi, f.lp_fmt, v);
+                    if (sig) {
+                        for (int j = k + 1; j <= depth; ++j) sig[j] = -2;
+                        sig[depth + 1] = (int)mask;
+                    }
+                }
             }
         }
-        if (k == depth) { ++k; break; }
-        const float u1 = pt_uniform(seed_h, texel, k, 0), u2 = pt_uniform(seed_h, texel, k, 1);
-        float sp, cp;
-        sincospif(2.0f * u2, &sp, &cp);
-        const float rr = sqrtf(u1);
-        const float lx = rr * cp, ly = rr * sp, lz = sqrtf(fmaxf(0.0f, 1.0f - u1));
-        const float sg = copysignf(1.0f, n.z);
-        const float aa = -1.0f / (sg + n.z);
-        const float bb = n.x * n.y * aa;
-        const float t1x = 1.0f + sg * n.x * n.x * aa, t1y = sg * bb, t1z = -sg * n.x;
-        const float t2x = bb, t2y = sg + n.y * n.y * aa, t2z = -n.y;
-        r.dx = fmaf(lx, t1x, fmaf(ly, t2x, lz * n.x));
-        r.dy = fmaf(lx, t1y, fmaf(ly, t2y, lz * n.y));
-        r.dz = fmaf(lx, t1z, fmaf(ly, t2z, lz * n.z));
-        r.ox = px; r.oy = py; r.oz = pz;
-        r.skip = h.id;
-        beta.x *= rho.x; beta.y *= rho.y; beta.z *= rho.z;
-    }
-    if (sig) {
-        for (; k <= depth; ++k) sig[k] = -2;
-        sig[depth + 1] = (int)mask;
-    }
-    return acc;
-}
-
-template <int TPB, int FETCH, int ORDER, class B>
-__global__ void __launch_bounds__(TPB)
-k_path_lp(const SceneDev sc, const __grid_constant__ B b, unsigned long long seed, int depth) {
-    const int lane = threadIdx.x & 31;
-    const unsigned long long seed_h = sm64_mix(seed);
-    while (true) {
-        unsigned long long base = 0ull;
-        if (lane == 0) base = atomicAdd(b.work_counter, (unsigned long long)FETCH);
-        base = __shfl_sync(0xffffffffu, base, 0);
-        if ((long long)base >= b.total_work) break;
-#pragma unroll 1
-        for (int k = 0; k < FETCH; k += 32) {
-            const long long w = (long long)base + k + lane;
-            if (w >= b.total_work) break;
-            const FrameDesc& f = b.d[find_frame(b, w, false)];
-            Ray r;
-            int glo, ghi;
-            const int local = (int)(w - f.work_begin);
-            const int t = lp_ray(f, local, r, glo, ghi);
-            const int col = __ldg(f.work + local).y;
-            const unsigned long long texel = (unsigned long long)(t - (2 * col + 1));  // oracle (compact) index
-            int* sig = f.hit_ids ? f.hit_ids + (long long)t * (depth + 2) : nullptr;
-            unsigned fault = 0u;
-            const float3 c = trace_path<ORDER>(sc, r, seed_h, texel, depth, sig, &fault);
-            if (fault) atomicOr(f.status, fault);
-            const float4 v = make_float4(c.x, c.y, c.z, 1.0f);
-            store_px(f.lp, t, f.lp_fmt, v);
-            if (glo >= 0) store_px(f.lp, glo, f.lp_fmt, v);
-            if (ghi >= 0) store_px(f.lp, ghi, f.lp_fmt, v);
+        __syncwarp();
+        const unsigned gm = __ballot_sync(full, go);
+        count -= n;
+        if (go) {
+            const int z = count + __popc(gm & ((1u << lane) - 1u));
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                P.o[c][z] = o[c];
+                P.d[c][z] = d[c];
+                __stcg(&S.beta[c][z], beta[c]);
+                __stcg(&S.acc[c][z], acc[c]);
+            }
+            __stcg(&S.cosl[z], cosl);
+            __stcg(&S.mask[z], mask);
+            P.skip[z] = skip;
+            P.work[z] = work;
+            P.step[z] = step;
         }
-    }
-}
-
-// Full-resolution path-traced GT: one path per display pixel centre (random
-// numbers keyed by the pixel index y W + x), written straight to the display.
-template <int TPB, int FETCH, int ORDER, class B>
-__global__ void __launch_bounds__(TPB)
-k_path_gt(const SceneDev sc, const __grid_constant__ B b, unsigned long long seed, int depth) {
-    const int lane = threadIdx.x & 31;
-    const unsigned long long seed_h = sm64_mix(seed);
-    while (true) {
-        unsigned long long base = 0ull;
-        if (lane == 0) base = atomicAdd(b.work_counter, (unsigned long long)FETCH);
-        base = __shfl_sync(0xffffffffu, base, 0);
-        if ((long long)base >= b.total_work) break;
-#pragma unroll 1
-        for (int k = 0; k < FETCH; k += 32) {
-            const long long w = (long long)base + k + lane;
-            if (w >= b.total_work) break;
-            const FrameDesc& f = b.d[find_frame(b, w, false)];
-            const long long local = w - f.work_begin;
-            const long long tile = local >> 5;
-            const int tiles_x = (f.W + 7) >> 3;
-            const int x = (int)(tile % tiles_x) * 8 + (lane & 7);
-            const int y = (int)(tile / tiles_x) * 4 + (lane >> 3);
-            if (x >= f.W || y >= f.H) continue;
-            const float cx = f.cr * ((float)x + 0.5f - 0.5f * (float)f.W);
-            const float cy = f.cr * (0.5f * (float)f.H - ((float)y + 0.5f));
-            Ray r;
-            world_ray(f, cx, cy, r);
-            const long long p = (long long)y * f.W + x;
-            unsigned fault = 0u;
-            const float3 c = trace_path<ORDER>(sc, r, seed_h, (unsigned long long)p, depth, nullptr, &fault);
-            if (fault) atomicOr(f.status, fault);
-            store_px(f.disp, p, f.disp_fmt, make_float4(c.x, c.y, c.z, 1.0f));
-        }
+        count += __popc(gm);
+        __syncwarp();
     }
 }
 
 template <bool GT, class B>
-cudaError_t launch_path_one(const SceneDev& sc, const B& b, unsigned long long seed, int depth, cudaStream_t s,
-                            int num_sms) {
+cudaError_t launch_path_one(const SceneDev& sc, const B& b, unsigned long long seed, int depth, void* scratch,
+                            cudaStream_t s, int num_sms) {
     if (b.total_work <= 0) return cudaSuccess;
-    constexpr int TPB = 128, FETCH = 32;
-    auto kern = GT ? k_path_gt<TPB, FETCH, 1, B> : k_path_lp<TPB, FETCH, 1, B>;
+    constexpr int TPB = 128;
+    auto kern = k_path<TPB, 0, GT, kPathBlocks, B>;
     int per_sm = 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, TPB, 0);
     if (e != cudaSuccess) return e;
-    if (per_sm < 1) per_sm = 1;
+    per_sm = min(max(per_sm, 1), kPathBlocks);   // the scratch holds this many blocks' pools
     e = cudaMemsetAsync(b.work_counter, 0, sizeof(unsigned long long), s);
     if (e != cudaSuccess) return e;
-    const long long want_warps = (b.total_work + FETCH - 1) / FETCH;
     long long grid = (long long)per_sm * num_sms;
-    const long long need = (want_warps * 32 + TPB - 1) / TPB;
+    const long long need = (b.total_work + TPB - 1) / TPB;
     if (need < grid) grid = need < 1 ? 1 : need;
-    kern<<<(unsigned)grid, TPB, 0, s>>>(sc, b, seed, depth);
+    kern<<<(unsigned)grid, TPB, 0, s>>>(sc, b, seed, depth, static_cast<PathState*>(scratch));
     count_launch(1);
     return cudaGetLastError();
 }
 }  // namespace
 
+size_t path_scratch_bytes(int num_sms) {
+    return sizeof(PathState) * (size_t)num_sms * kPathBlocks * 4;
+}
+
 template <class B>
 cudaError_t launch_path_lp(const SceneDev& scene, const B& batch, unsigned long long seed, int depth,
-                           cudaStream_t s, int num_sms) {
-    return launch_path_one<false>(scene, batch, seed, depth, s, num_sms);
+                           void* scratch, cudaStream_t s, int num_sms) {
+    return launch_path_one<false>(scene, batch, seed, depth, scratch, s, num_sms);
 }
 template <class B>
 cudaError_t launch_path_gt(const SceneDev& scene, const B& batch, unsigned long long seed, int depth,
-                           cudaStream_t s, int num_sms) {
-    return launch_path_one<true>(scene, batch, seed, depth, s, num_sms);
+                           void* scratch, cudaStream_t s, int num_sms) {
+    return launch_path_one<true>(scene, batch, seed, depth, scratch, s, num_sms);
 }
-template cudaError_t launch_path_gt<SmallBatch>(const SceneDev&, const SmallBatch&, unsigned long long, int,
+template cudaError_t launch_path_gt<SmallBatch>(const SceneDev&, const SmallBatch&, unsigned long long, int, void*,
                                                 cudaStream_t, int);
-template cudaError_t launch_path_lp<SmallBatch>(const SceneDev&, const SmallBatch&, unsigned long long, int,
+template cudaError_t launch_path_lp<SmallBatch>(const SceneDev&, const SmallBatch&, unsigned long long, int, void*,
                                                 cudaStream_t, int);
-template cudaError_t launch_path_lp<BigBatch>(const SceneDev&, const BigBatch&, unsigned long long, int,
+template cudaError_t launch_path_lp<BigBatch>(const SceneDev&, const BigBatch&, unsigned long long, int, void*,
                                               cudaStream_t, int);
 
 }  // namespace vafr

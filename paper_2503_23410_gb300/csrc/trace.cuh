@@ -287,10 +287,11 @@ __device__ __forceinline__ unsigned child_key(float t, unsigned word) {
 // slot that any lane needs); the closest-hit rule (t, then id) makes the
 // result independent of the order.
 // Returns a fault bit (0 = fine).
-template <bool STATS, int ORDER, bool ANY = false, bool SKIP = false>
-__device__ unsigned traverse4(const SceneDev& sc, const Ray& r, Hit& h,
-                              unsigned long long* node_visits, unsigned long long* box_tests,
-                              unsigned long long* tri_tests) {
+// `any`: an occlusion query, which ends at the first hit found.
+template <bool STATS, int ORDER, bool SKIP = false>
+__device__ __forceinline__ unsigned traverse4(const SceneDev& sc, const Ray& r, Hit& h,
+                                              unsigned long long* node_visits, unsigned long long* box_tests,
+                                              unsigned long long* tri_tests, bool any = false) {
     h.t = INFINITY;
     h.leaf = -1;
     h.id = INT_MAX;
@@ -337,7 +338,7 @@ __device__ unsigned traverse4(const SceneDev& sc, const Ray& r, Hit& h,
             if ((unsigned)~C >= (unsigned)sc.n_tris) return kFaultBadNode;
             test_leaf<STATS, SKIP>(sc, r, ~C, h, tri_tests);
         }
-        if (ANY && h.leaf >= 0) return 0u;   // occlusion query: any hit ends it
+        if (any && h.leaf >= 0) return 0u;
         // children entering beyond a closest hit found at this node are dropped
         // (the box tests already clipped against the hit known before it)
         if (h.t != t_entry) {

@@ -157,12 +157,14 @@ template <class B>
 cudaError_t launch_reconstruct(const B& batch, int variant, cudaStream_t s);
 // Path-traced LP buffers (pathtrace.cu): one path per texel, `depth` diffuse
 // bounces; FrameDesc.hit_ids, when set, receives depth + 2 ints per slot.
+// `scratch` holds path_scratch_bytes device bytes of the launch's own.
+size_t path_scratch_bytes(int num_sms);
 template <class B>
 cudaError_t launch_path_lp(const SceneDev& scene, const B& batch, unsigned long long seed, int depth,
-                           cudaStream_t s, int num_sms);
+                           void* scratch, cudaStream_t s, int num_sms);
 template <class B>
 cudaError_t launch_path_gt(const SceneDev& scene, const B& batch, unsigned long long seed, int depth,
-                           cudaStream_t s, int num_sms);
+                           void* scratch, cudaStream_t s, int num_sms);
 // Ray casting of an explicit list of (slot, column) work items whose count
 // is read from device memory (render.cu): the reprojection's holes.
 cudaError_t launch_render_list(const SceneDev& scene, const SmallBatch& batch, const unsigned* count,
