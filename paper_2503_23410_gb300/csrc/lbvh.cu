@@ -4,9 +4,11 @@
 //   2. 30-bit Morton codes of s on a cubic grid of 1024 cells along the
 //      largest extent of the bounds,
 //   3. stable LSD radix sort of (code, triangle id), 4 passes of 8 bits,
-//   4. binary radix tree: one thread per internal node,
-//   5. bottom-up FP32 bounds with one arrival counter per internal node,
-//   6. packing into the 64-byte two-child traversal node + 48-byte leaves.
+//   4. sorted leaves: triangle box, 48-byte traversal leaf, the traversal
+//      tree's first clusters,
+//   5. binary radix tree: one thread per internal node,
+//   6. bottom-up FP32 bounds, a node's second arrival writing its box and its
+//      64-byte two-child traversal node.
 // The quantisation uses explicitly rounded intrinsics (no FMA contraction) so
 // the codes are bit-identical to any IEEE FP32 evaluation of the same sequence.
 // No kernel here waits on another thread: there is nothing that can spin.
@@ -20,6 +22,9 @@
 #include <mutex>
 
 namespace vafr {
+
+size_t lbvh_sort_blocks(int n);
+
 namespace {
 
 constexpr int kSortThreads = 256;
@@ -65,12 +70,16 @@ __global__ void k_bounds_partial(const float* __restrict__ tris, int n, float* _
     }
 }
 
+// One warp per bound (a minimum or maximum over the blocks' partial bounds).
 __global__ void k_bounds_final(const float* __restrict__ part, int nb, float* __restrict__ out) {
-    const int k = threadIdx.x;
-    if (k >= 6) return;
+    const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
     float v = part[k];
-    for (int b = 1; b < nb; ++b) v = k < 3 ? fminf(v, part[6 * b + k]) : fmaxf(v, part[6 * b + k]);
-    out[k] = v;
+    for (int b = lane; b < nb; b += 32) v = k < 3 ? fminf(v, part[6 * b + k]) : fmaxf(v, part[6 * b + k]);
+    for (int o = 16; o > 0; o >>= 1) {
+        const float w = __shfl_xor_sync(0xffffffffu, v, o);
+        v = k < 3 ? fminf(v, w) : fmaxf(v, w);
+    }
+    if (lane == 0) out[k] = v;
 }
 
 // 10 bits spread to every third bit position (bit b -> bit 3b).
@@ -123,45 +132,69 @@ __global__ void k_radix_hist(const uint32_t* __restrict__ keys, int n, int shift
         if (i < n) atomicAdd(&h[(keys[i] >> shift) & 255u], 1u);
     }
     __syncthreads();
-    hist[threadIdx.x * nblocks + blockIdx.x] = h[threadIdx.x];
+    hist[(size_t)threadIdx.x * nblocks + blockIdx.x] = h[threadIdx.x];
 }
 
-// Exclusive scan of `total` counters by one block of 1024 threads.
-__global__ void k_radix_scan(unsigned* __restrict__ hist, int total) {
-    __shared__ unsigned part[1024];
-    const int per = (total + 1023) / 1024;
-    const int b = threadIdx.x * per;
-    unsigned s = 0;
-    for (int i = 0; i < per; ++i)
-        if (b + i < total) s += hist[b + i];
-    part[threadIdx.x] = s;
-    __syncthreads();
-    for (int o = 1; o < 1024; o <<= 1) {
-        unsigned v = threadIdx.x >= (unsigned)o ? part[threadIdx.x - o] : 0u;
-        __syncthreads();
-        part[threadIdx.x] += v;
-        __syncthreads();
-    }
-    unsigned run = part[threadIdx.x] - s;   // exclusive prefix of this chunk
-    for (int i = 0; i < per; ++i) {
-        if (b + i < total) {
-            unsigned v = hist[b + i];
-            hist[b + i] = run;
-            run += v;
+// Block d scans digit d's counters over the tiles (exclusive, in place) and
+// leaves their sum in total[d]; the scatter adds the smaller digits' totals.
+// A single block scanning all 256 x tiles counters took 110 us of each pass at
+// 1.07 M keys (134 K counters); 256 blocks take 4 us.
+__global__ void __launch_bounds__(kSortThreads) k_radix_rows(unsigned* __restrict__ hist, int nblocks,
+                                                             unsigned* __restrict__ total) {
+    __shared__ unsigned warp_sum[kSortWarps];
+    unsigned* row = hist + (size_t)blockIdx.x * nblocks;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    unsigned carry = 0u;
+    for (int base = 0; base < nblocks; base += kSortThreads) {
+        const int i = base + (int)threadIdx.x;
+        const unsigned x = i < nblocks ? row[i] : 0u;
+        unsigned incl = x;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
         }
+        if (lane == 31) warp_sum[warp] = incl;
+        __syncthreads();
+        unsigned before = 0u, all = 0u;
+#pragma unroll
+        for (int w = 0; w < kSortWarps; ++w) {
+            const unsigned c = warp_sum[w];
+            before += w < warp ? c : 0u;
+            all += c;
+        }
+        if (i < nblocks) row[i] = carry + before + incl - x;
+        carry += all;
+        __syncthreads();
     }
+    if (threadIdx.x == 0) total[blockIdx.x] = carry;
 }
 
 __global__ void __launch_bounds__(kSortThreads)
 k_radix_scatter(const uint32_t* __restrict__ kin, const int32_t* __restrict__ vin,
                 uint32_t* __restrict__ kout, int32_t* __restrict__ vout, int n, int shift,
-                const unsigned* __restrict__ hist, int nblocks) {
+                const unsigned* __restrict__ hist, int nblocks, const unsigned* __restrict__ total) {
     __shared__ unsigned cnt[kSortWarps][256];
     __shared__ unsigned gbase[256];
-    for (int i = threadIdx.x; i < kSortWarps * 256; i += kSortThreads) (&cnt[0][0])[i] = 0u;
-    gbase[threadIdx.x] = hist[threadIdx.x * nblocks + blockIdx.x];
-    __syncthreads();
+    __shared__ unsigned warp_sum[kSortWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int i = threadIdx.x; i < kSortWarps * 256; i += kSortThreads) (&cnt[0][0])[i] = 0u;
+    {   // first slot of this tile's keys with digit threadIdx.x
+        const unsigned x = total[threadIdx.x];
+        unsigned incl = x;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        if (lane == 31) warp_sum[warp] = incl;
+        __syncthreads();
+        unsigned before = 0u;
+#pragma unroll
+        for (int w = 0; w < kSortWarps; ++w) before += w < warp ? warp_sum[w] : 0u;
+        gbase[threadIdx.x] = before + incl - x + hist[(size_t)threadIdx.x * nblocks + blockIdx.x];
+    }
+    __syncthreads();
     const unsigned lt = (1u << lane) - 1u;
     const long long base = (long long)blockIdx.x * kSortTile + (long long)warp * (32 * kSortItems);
     uint32_t key[kSortItems];
@@ -216,8 +249,11 @@ __device__ __forceinline__ int delta(const uint32_t* __restrict__ k, int n, int 
     return __clz(ki ^ kj);
 }
 
+// links[i] = (left, right, other end of node i's leaves, parent): what a climb
+// needs of a node in one load.  A node's thread writes all but the parent,
+// which its parent's thread writes.
 __global__ void k_karras(const uint32_t* __restrict__ keys, int n, int2* __restrict__ child,
-                         int32_t* __restrict__ parent) {
+                         int4* __restrict__ links, int32_t* __restrict__ leaf_parent) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n - 1) return;
     const uint32_t ki = keys[i];
@@ -240,9 +276,11 @@ __global__ void k_karras(const uint32_t* __restrict__ keys, int n, int2* __restr
     const int L = (lo == gamma) ? ~gamma : gamma;
     const int R = (hi == gamma + 1) ? ~(gamma + 1) : gamma + 1;
     child[i] = make_int2(L, R);
-    parent[L >= 0 ? L : (n - 1) + ~L] = i;
-    parent[R >= 0 ? R : (n - 1) + ~R] = i;
-    if (i == 0) parent[0] = -1;
+    *reinterpret_cast<int2*>(&links[i]) = make_int2(L, R);
+    links[i].z = j;
+    *(L >= 0 ? &links[L].w : &leaf_parent[~L]) = i;
+    *(R >= 0 ? &links[R].w : &leaf_parent[~R]) = i;
+    if (i == 0) links[0].w = -1;
 }
 
 __device__ __forceinline__ void load_box(const float* p, float b[6]) {
@@ -250,78 +288,159 @@ __device__ __forceinline__ void load_box(const float* p, float b[6]) {
     for (int k = 0; k < 6; ++k) b[k] = __ldcg(p + k);
 }
 
-// Bottom-up bounds: each leaf thread writes its box and climbs; at every
-// internal node the first arrival stops and the second (which then sees both
-// children's boxes) writes the union and continues.
-__global__ void k_refit(const float* __restrict__ tris, const int32_t* __restrict__ ids, int n,
-                        const int2* __restrict__ child, const int32_t* __restrict__ parent,
-                        unsigned* __restrict__ flags, float* __restrict__ node_box,
-                        float* __restrict__ leaf_box) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n) return;
-    const float* t = tris + 9ll * ids[k];
+__device__ __forceinline__ void merge_box(float b[6], const float a[6]) {
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        leaf_box[6ll * k + a] = fminf(fminf(t[a], t[3 + a]), t[6 + a]);
-        leaf_box[6ll * k + 3 + a] = fmaxf(fmaxf(t[a], t[3 + a]), t[6 + a]);
-    }
-    if (n == 1) return;
-    int node = parent[(n - 1) + k];
-    // a binary radix tree over 30-bit codes + 32-bit positions is at most 64
-    // levels deep; the bound only guards against a malformed parent array
-    for (int climb = 0; node >= 0 && climb < 96; ++climb) {
-        __threadfence();
-        if (atomicAdd(&flags[node], 1u) == 0u) return;
-        __threadfence();
-        const int2 c = child[node];
-        float a[6], b[6];
-        load_box(c.x >= 0 ? node_box + 6ll * c.x : leaf_box + 6ll * ~c.x, a);
-        load_box(c.y >= 0 ? node_box + 6ll * c.y : leaf_box + 6ll * ~c.y, b);
-        float* o = node_box + 6ll * node;
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            __stcg(o + q, fminf(a[q], b[q]));
-            __stcg(o + 3 + q, fmaxf(a[3 + q], b[3 + q]));
-        }
-        node = parent[node];
+    for (int q = 0; q < 3; ++q) {
+        b[q] = fminf(b[q], a[q]);
+        b[3 + q] = fmaxf(b[3 + q], a[3 + q]);
     }
 }
 
-__global__ void k_pack_nodes(const int2* __restrict__ child, const float* __restrict__ node_box,
-                             const float* __restrict__ leaf_box, int n, float4* __restrict__ nodes) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n - 1) return;
-    const int2 c = child[i];
-    const float* a = c.x >= 0 ? node_box + 6ll * c.x : leaf_box + 6ll * ~c.x;
-    const float* b = c.y >= 0 ? node_box + 6ll * c.y : leaf_box + 6ll * ~c.y;
-    // per axis: (left lo, right lo, left hi, right hi), so both children's slabs
-    // are computed with paired FP32 instructions
-    nodes[4ll * i + 0] = make_float4(a[0], b[0], a[3], b[3]);
-    nodes[4ll * i + 1] = make_float4(a[1], b[1], a[4], b[4]);
-    nodes[4ll * i + 2] = make_float4(a[2], b[2], a[5], b[5]);
-    nodes[4ll * i + 3] = make_float4(__int_as_float(c.x), __int_as_float(c.y), 0.0f, 0.0f);
+// Bottom-up bounds: a thread per leaf climbs; at every internal node the first
+// arrival stops and the second, which then has both children's boxes, writes
+// the node's box and its two-child traversal node and continues.
+// In k_refit_block a block takes kRefitLeaves consecutive leaves and makes the
+// nodes whose leaves all lie among them: the children meet in shared memory.
+// The few nodes above, one in some hundred, are left to k_refit_top, which
+// climbs on from the listed children; there each arrival costs a device-wide
+// fence and an atomic.  (One kernel for both kept a block's place on its SM
+// for as long as its last thread climbed to the top: 143 us at 1.07 M leaves;
+// every node in global memory and the traversal nodes packed in a pass of
+// their own 176 us; the two kernels 69 + 52 us.)
+constexpr int kRefitLeaves = 512;
+
+// A child whose parent is the next to be made: box b, its sibling's box a.
+__device__ __forceinline__ void make_parent(int node, int2 kids, int side, float b[6], const float a[6],
+                                            float* __restrict__ node_box, float4* __restrict__ nodes) {
+    float L[6], R[6];
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {
+        L[q] = side ? a[q] : b[q];
+        R[q] = side ? b[q] : a[q];
+    }
+    // per axis: (left lo, right lo, left hi, right hi), so both children's
+    // slabs are computed with paired FP32 instructions
+    float4* nd = nodes + 4ll * node;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) nd[q] = make_float4(L[q], R[q], L[q + 3], R[q + 3]);
+    nd[3] = make_float4(__int_as_float(kids.x), __int_as_float(kids.y), 0.0f, 0.0f);
+    merge_box(b, a);
+    float* o = node_box + 6ll * node;
+#pragma unroll
+    for (int q = 0; q < 6; ++q) __stcg(o + q, b[q]);
+}
+
+__global__ void __launch_bounds__(kRefitLeaves)
+k_refit_block(int n, const int4* __restrict__ links, const int32_t* __restrict__ leaf_parent,
+              float* __restrict__ node_box, const float* __restrict__ leaf_box, float4* __restrict__ nodes,
+              int* __restrict__ list, unsigned* __restrict__ listed) {
+    __shared__ unsigned met[kRefitLeaves];
+    __shared__ float box[2][6][kRefitLeaves];   // [child side][bound][node - b0]
+    __shared__ int4 link[kRefitLeaves];
+    __shared__ int up[kRefitLeaves];            // children whose parent has other leaves too
+    __shared__ unsigned ups, at;
+    const int b0 = (int)blockIdx.x * kRefitLeaves;
+    const int k = b0 + (int)threadIdx.x;
+    met[threadIdx.x] = 0u;
+    if (threadIdx.x == 0) ups = 0u;
+    if (k < n - 1) link[threadIdx.x] = links[k];
+    __syncthreads();
+    if (k < n) {
+        float b[6];
+        load_box(leaf_box + 6ll * k, b);
+        int ref = ~k;
+        int node = leaf_parent[k];
+        while (node >= 0) {
+            const int s = node - b0;   // a node's index is one end of its leaves
+            if ((unsigned)s >= (unsigned)kRefitLeaves || (unsigned)(link[s].z - b0) >= (unsigned)kRefitLeaves) {
+                const unsigned q = atomicAdd(&ups, 1u);   // a leaf's thread gets here at most once
+                up[q] = ref;
+                break;
+            }
+            const int2 c = make_int2(link[s].x, link[s].y);
+            const int side = c.x == ref ? 0 : 1;
+#pragma unroll
+            for (int q = 0; q < 6; ++q) box[side][q][s] = b[q];
+            __threadfence_block();
+            if (atomicAdd(&met[s], 1u) != 1u) break;   // the first arrival; anything else only in a malformed tree
+            __threadfence_block();
+            float a[6];
+#pragma unroll
+            for (int q = 0; q < 6; ++q) a[q] = *(volatile float*)&box[side ^ 1][q][s];
+            make_parent(node, c, side, b, a, node_box, nodes);
+            ref = node;
+            node = link[s].w;
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) at = ups ? atomicAdd(listed, ups) : 0u;
+    __syncthreads();
+    if (threadIdx.x < ups) list[at + threadIdx.x] = up[threadIdx.x];
+}
+
+__global__ void __launch_bounds__(256)
+k_refit_top(int n, const int4* __restrict__ links, const int32_t* __restrict__ leaf_parent,
+            unsigned* __restrict__ flags, float* __restrict__ node_box, const float* __restrict__ leaf_box,
+            float4* __restrict__ nodes, const int* __restrict__ list, const unsigned* __restrict__ listed) {
+    const unsigned count = min(*listed, (unsigned)n);
+    for (unsigned q = blockIdx.x * 256 + threadIdx.x; q < count; q += gridDim.x * 256) {
+        int ref = list[q];
+        float b[6];
+        load_box(ref >= 0 ? node_box + 6ll * ref : leaf_box + 6ll * ~ref, b);
+        int node = ref >= 0 ? links[ref].w : leaf_parent[~ref];
+        // a binary radix tree over 30-bit codes + 32-bit positions is at most 64
+        // levels deep; the bound only guards against a malformed parent array
+        int4 next = node >= 0 ? links[node] : make_int4(0, 0, 0, -1);
+        for (int climb = 0; node >= 0 && climb < 96; ++climb) {
+            const int4 ln = next;
+            if (ln.w >= 0) next = links[ln.w];   // on its way while the arrival is counted
+            __threadfence();   // this child's box, if written here, before its arrival
+            if (atomicAdd(&flags[node], 1u) == 0u) break;
+            __threadfence();
+            const int2 c = make_int2(ln.x, ln.y);
+            const int side = c.x == ref ? 0 : 1;
+            const int sib = side ? c.x : c.y;
+            float a[6];
+            load_box(sib >= 0 ? node_box + 6ll * sib : leaf_box + 6ll * ~sib, a);
+            make_parent(node, c, side, b, a, node_box, nodes);
+            ref = node;
+            node = ln.w;
+        }
+    }
 }
 
 __device__ __forceinline__ bool lex_less(float ax, float ay, float az, float bx, float by, float bz) {
     return ax < bx || (ax == bx && (ay < by || (ay == by && az < bz)));
 }
 
+// Sorted leaf k: its triangle's box, its traversal leaf, and the cluster that
+// the traversal tree starts from (box with the reference ~k in lo.w).
 // Leaves store their vertices in lexicographic (x, y, z) order.  The
 // intersection test is two-sided, so the order carries no meaning, and
 // identical triangles given with different vertex orders then evaluate to
 // bit-identical t: the lower-id rule, not rounding, decides between them.
-__global__ void k_pack_leaves(const float* __restrict__ tris, const float* __restrict__ albedo,
-                              const int32_t* __restrict__ ids, int n, float4* __restrict__ leaves,
-                              float4* __restrict__ albedo4) {
+__global__ void k_leaves(const float* __restrict__ tris, const float* __restrict__ albedo,
+                         const int32_t* __restrict__ ids, int n, float* __restrict__ leaf_box,
+                         float4* __restrict__ leaves, float4* __restrict__ clusters,
+                         float4* __restrict__ albedo4) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n) return;
     const int id = ids[k];
     const float* t = tris + 9ll * id;
-    float v[3][3];
+    float v[3][3], lo[3], hi[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a)
 #pragma unroll
         for (int c = 0; c < 3; ++c) v[a][c] = t[3 * a + c];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        lo[c] = fminf(fminf(v[0][c], v[1][c]), v[2][c]);
+        hi[c] = fmaxf(fmaxf(v[0][c], v[1][c]), v[2][c]);
+        leaf_box[6ll * k + c] = lo[c];
+        leaf_box[6ll * k + 3 + c] = hi[c];
+    }
+    clusters[2ll * k] = make_float4(lo[0], lo[1], lo[2], __int_as_float(~k));
+    clusters[2ll * k + 1] = make_float4(hi[0], hi[1], hi[2], 0.0f);
     // three-element sorting network
 #define VAFR_CSWAP(i, j)                                                                      \
     if (lex_less(v[j][0], v[j][1], v[j][2], v[i][0], v[i][1], v[i][2])) {                     \
@@ -343,49 +462,61 @@ __global__ void k_pack_leaves(const float* __restrict__ tris, const float* __res
 
 inline int blocks_for(long long n, int tpb) { return (int)((n + tpb - 1) / tpb); }
 
-}  // namespace
-
-size_t lbvh_sort_blocks(int n) { return (size_t)((n + kSortTile - 1) / kSortTile); }
-
-cudaError_t lbvh_build(const LbvhBuffers& b, cudaStream_t s) {
-    const int n = b.n;
-    if (n <= 0) return cudaSuccess;
+// Morton codes of the triangles, then the stable (code, id) order: codes in
+// input order stay in `codes`, the sorted keys and ids end in `keys` and `ids`.
+// `hist` holds 256 counters per tile and 256 totals.
+void morton_sort(const float* tris, int n, float* part_bounds, float* scene_bounds, uint32_t* codes,
+                 uint32_t* keys_tmp, int32_t* ids_tmp, uint32_t* keys, int32_t* ids, unsigned* hist, cudaStream_t s) {
     const int nb_bounds = min(kBoundsBlocks, blocks_for(n, 256));
-    k_bounds_partial<<<nb_bounds, 256, 0, s>>>(b.tris, n, b.part_bounds);
-    k_bounds_final<<<1, 32, 0, s>>>(b.part_bounds, nb_bounds, b.scene_bounds);
-    k_morton<<<blocks_for(n, 256), 256, 0, s>>>(b.tris, n, b.scene_bounds, b.codes);
+    k_bounds_partial<<<nb_bounds, 256, 0, s>>>(tris, n, part_bounds);
+    k_bounds_final<<<1, 192, 0, s>>>(part_bounds, nb_bounds, scene_bounds);
+    k_morton<<<blocks_for(n, 256), 256, 0, s>>>(tris, n, scene_bounds, codes);
     count_launch(3);
     const int nblocks = (int)lbvh_sort_blocks(n);
+    unsigned* total = hist + 256ull * nblocks;
     // ping-pong: codes -> tmp -> sorted -> tmp -> sorted
-    const uint32_t* kin = b.codes;
+    const uint32_t* kin = codes;
     const int32_t* vin = nullptr;
     for (int pass = 0; pass < 4; ++pass) {
-        uint32_t* kout = (pass & 1) ? b.keys_sorted : b.keys_tmp;
-        int32_t* vout = (pass & 1) ? b.ids : b.ids_tmp;
-        k_radix_hist<<<nblocks, kSortThreads, 0, s>>>(kin, n, 8 * pass, b.hist, nblocks);
-        k_radix_scan<<<1, 1024, 0, s>>>(b.hist, 256 * nblocks);
-        k_radix_scatter<<<nblocks, kSortThreads, 0, s>>>(kin, vin, kout, vout, n, 8 * pass,
-                                                         b.hist, nblocks);
+        uint32_t* kout = (pass & 1) ? keys : keys_tmp;
+        int32_t* vout = (pass & 1) ? ids : ids_tmp;
+        k_radix_hist<<<nblocks, kSortThreads, 0, s>>>(kin, n, 8 * pass, hist, nblocks);
+        k_radix_rows<<<256, kSortThreads, 0, s>>>(hist, nblocks, total);
+        k_radix_scatter<<<nblocks, kSortThreads, 0, s>>>(kin, vin, kout, vout, n, 8 * pass, hist, nblocks, total);
         count_launch(3);
         kin = kout;
         vin = vout;
     }
-    if (n > 1) {
-        cudaMemsetAsync(b.flags, 0, sizeof(unsigned) * (size_t)(n - 1), s);
-        k_karras<<<blocks_for(n - 1, 256), 256, 0, s>>>(b.keys_sorted, n, b.child, b.parent);
-        count_launch(1);
-    }
-    k_refit<<<blocks_for(n, 256), 256, 0, s>>>(b.tris, b.ids, n, b.child, b.parent, b.flags,
-                                               b.node_box, b.leaf_box);
+}
+
+}  // namespace
+
+size_t lbvh_sort_blocks(int n) { return (size_t)((n + kSortTile - 1) / kSortTile); }
+size_t lbvh_hist_elems(int n) { return 256 * (lbvh_sort_blocks(n) + 1); }
+
+cudaError_t lbvh_sort(const LbvhBuffers& b, cudaStream_t s) {
+    const int n = b.n;
+    if (n <= 0) return cudaSuccess;
+    morton_sort(b.tris, n, b.part_bounds, b.scene_bounds, b.codes, b.keys_tmp, b.ids_tmp, b.keys_sorted, b.ids,
+                b.hist, s);
+    k_leaves<<<blocks_for(n, 256), 256, 0, s>>>(b.tris, b.albedo, b.ids, n, b.leaf_box, b.leaves, b.clusters,
+                                                b.albedo4);
     count_launch(1);
-    if (n > 1) {
-        k_pack_nodes<<<blocks_for(n - 1, 256), 256, 0, s>>>(b.child, b.node_box, b.leaf_box, n,
-                                                            b.nodes);
-        count_launch(1);
-    }
-    k_pack_leaves<<<blocks_for(n, 256), 256, 0, s>>>(b.tris, b.albedo, b.ids, n, b.leaves,
-                                                     b.albedo4);
-    count_launch(1);
+    return cudaGetLastError();
+}
+
+cudaError_t lbvh_hierarchy(const LbvhBuffers& b, cudaStream_t s) {
+    const int n = b.n;
+    if (n <= 1) return cudaSuccess;
+    cudaError_t e = cudaMemsetAsync(b.flags, 0, sizeof(unsigned) * (size_t)n, s);   // n - 1 nodes, the list's length
+    if (e != cudaSuccess) return e;
+    unsigned* listed = b.flags + (n - 1);
+    k_karras<<<blocks_for(n - 1, 256), 256, 0, s>>>(b.keys_sorted, n, b.child, b.links, b.leaf_parent);
+    k_refit_block<<<blocks_for(n, kRefitLeaves), kRefitLeaves, 0, s>>>(n, b.links, b.leaf_parent, b.node_box,
+                                                                       b.leaf_box, b.nodes, b.climbers, listed);
+    k_refit_top<<<min(blocks_for(n, 256), 304), 256, 0, s>>>(n, b.links, b.leaf_parent, b.flags, b.node_box, b.leaf_box,
+                                                             b.nodes, b.climbers, listed);
+    count_launch(3);
     return cudaGetLastError();
 }
 
@@ -407,7 +538,7 @@ struct NoAllocScratch {
     uint32_t keys_tmp[kNoAllocMaxTris];
     int32_t ids_tmp[kNoAllocMaxTris];
     uint32_t keys_sorted[kNoAllocMaxTris];
-    unsigned hist[256 * kNoAllocBlocks];
+    unsigned hist[256 * (kNoAllocBlocks + 1)];
     float part_bounds[6 * kBoundsBlocks];
     float scene_bounds[8];
 };
@@ -517,25 +648,8 @@ extern "C" VAFR_API int vafr_morton_sort_noalloc(const float* tri_xyz, int64_t n
     if (e != cudaSuccess) return report(VAFR_ERR_CUDA, cudaGetErrorString(e));
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     const int n = (int)n_tris;
-    const int nb_bounds = min(kBoundsBlocks, blocks_for(n, 256));
-    k_bounds_partial<<<nb_bounds, 256, 0, s>>>(tri_xyz, n, sc->part_bounds);
-    k_bounds_final<<<1, 32, 0, s>>>(sc->part_bounds, nb_bounds, sc->scene_bounds);
-    k_morton<<<blocks_for(n, 256), 256, 0, s>>>(tri_xyz, n, sc->scene_bounds, codes_out);
-    count_launch(3);
-    const int nblocks = (int)lbvh_sort_blocks(n);
-    const uint32_t* kin = codes_out;
-    const int32_t* vin = nullptr;
-    for (int pass = 0; pass < 4; ++pass) {
-        uint32_t* kout = (pass & 1) ? sc->keys_sorted : sc->keys_tmp;
-        int32_t* vout = (pass & 1) ? sorted_ids_out : sc->ids_tmp;
-        k_radix_hist<<<nblocks, kSortThreads, 0, s>>>(kin, n, 8 * pass, sc->hist, nblocks);
-        k_radix_scan<<<1, 1024, 0, s>>>(sc->hist, 256 * nblocks);
-        k_radix_scatter<<<nblocks, kSortThreads, 0, s>>>(kin, vin, kout, vout, n, 8 * pass,
-                                                         sc->hist, nblocks);
-        count_launch(3);
-        kin = kout;
-        vin = vout;
-    }
+    morton_sort(tri_xyz, n, sc->part_bounds, sc->scene_bounds, codes_out, sc->keys_tmp, sc->ids_tmp, sc->keys_sorted,
+                sorted_ids_out, sc->hist, s);
     e = cudaGetLastError();
     if (e != cudaSuccess) return report(VAFR_ERR_CUDA, cudaGetErrorString(e));
     return VAFR_OK;

@@ -203,42 +203,53 @@ cudaError_t launch_fxaa(const B& batch, cudaStream_t s, int num_sms);
 cudaError_t launch_render_stats(const SceneDev& scene, const SmallBatch& batch,
                                 unsigned long long* counters, cudaStream_t s, int num_sms);
 
-// LBVH build (lbvh.cu).  All device pointers are owned by the caller.
+// Scene build.  All device pointers are owned by the caller.  The steps run in
+// this order, and the caller lays their scratch out so that each step's takes
+// the place of the earlier ones':
+//   lbvh_sort       Morton codes, their order, the sorted leaves (lbvh.cu)
+//   tree4_build     traversal tree: PLOC over the sorted leaves, collapsed to
+//                   4-wide nodes, which it numbers and counts (tree4.cu;
+//                   synchronises `s` to read the count)
+//   tree4_pack      ... written to b.nodes4 (16 float4 per node), which the
+//                   caller allocates after tree4_build
+//   lbvh_hierarchy  binary radix tree over the sorted codes and its bounds
 struct LbvhBuffers {
     const float* tris;      // n x 9 input (device)
     const float* albedo;    // n x 3 (device) or nullptr
     int n;
+    // what the scene keeps
     uint32_t* codes;        // n  Morton codes, input order
-    uint32_t* keys_tmp;     // n  sort scratch
     int32_t* ids;           // n  sorted triangle ids
-    int32_t* ids_tmp;       // n  sort scratch
-    uint32_t* keys_sorted;  // n
-    unsigned* hist;         // 256 * blocks
-    float* part_bounds;     // 6 * blocks
-    float* scene_bounds;    // 6
-    int2* child;            // n-1
-    int32_t* parent;        // (n-1) + n: parents of internal nodes then leaves
-    unsigned* flags;        // n-1 refit arrival counters
-    float* node_box;        // (n-1) x 6
     float* leaf_box;        // n x 6
-    float4* nodes;          // (n-1) x 4
-    unsigned* head_flag;    // n-1: internal node at even depth
-    unsigned* head_idx;     // n-1: its 4-wide node index (each node's internal children consecutive)
-    float4* nodes4;         // n_nodes4 x 16 (allocated once tree4_build has counted them)
     float4* leaves;         // n x 3
     float4* albedo4;        // n
+    float4* nodes4;         // n_nodes4 x 16
+    int2* child;            // n-1, written by lbvh_hierarchy
+    float* node_box;        // (n-1) x 6, written by lbvh_hierarchy
+    float4* nodes;          // (n-1) x 4, written by lbvh_hierarchy
+    // from lbvh_sort to lbvh_hierarchy
+    uint32_t* keys_sorted;  // n
+    // within lbvh_sort
+    uint32_t* keys_tmp;     // n
+    int32_t* ids_tmp;       // n
+    unsigned* hist;         // lbvh_hist_elems(n)
+    float* part_bounds;     // 6 * 304
+    float* scene_bounds;    // 6
+    // from lbvh_sort to tree4_build
+    float4* clusters;       // n x 2: leaf boxes with their references
+    // within lbvh_hierarchy
+    int4* links;            // n-1: each internal node's children, the other end of its leaves, its parent
+    int32_t* leaf_parent;   // n
+    unsigned* flags;        // n: arrival counters of the nodes, then the length of `climbers`
+    int32_t* climbers;      // n: children whose parents are made last
 };
 size_t lbvh_sort_blocks(int n);
-cudaError_t lbvh_build(const LbvhBuffers& b, cudaStream_t s);
-// Traversal tree (tree4.cu): PLOC over the sorted leaves, collapsed to
-// 4-wide nodes.  tree4_build clusters, numbers the nodes and returns their
-// count; the caller allocates b.nodes4 (16 float4 per node) and tree4_pack
-// writes them.  `scratch` holds tree4_scratch_bytes(n) device bytes, carries
-// the binary tree from the first call to the second and may be freed after
-// it (both synchronise `s`).
-constexpr int kPlocRadius = 8;
+size_t lbvh_hist_elems(int n);
+cudaError_t lbvh_sort(const LbvhBuffers& b, cudaStream_t s);
+cudaError_t lbvh_hierarchy(const LbvhBuffers& b, cudaStream_t s);
+// `scratch`: tree4_scratch_bytes(n) device bytes, from tree4_build to tree4_pack.
 size_t tree4_scratch_bytes(int n);
-cudaError_t tree4_build(const LbvhBuffers& b, void* scratch, int radius, cudaStream_t s, int* n_nodes4);
+cudaError_t tree4_build(const LbvhBuffers& b, void* scratch, cudaStream_t s, int num_sms, int* n_nodes4);
 cudaError_t tree4_pack(const LbvhBuffers& b, void* scratch, int n_nodes4, cudaStream_t s);
 
 // FP32 issue rate (peak.cu): FMAs per second of scalar FFMA and of paired
