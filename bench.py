@@ -70,7 +70,7 @@ PT_DIFFUSE = 3        # the paper's maximum diffuse bounces (Sec. 8.1)
 # is the pixel ray (15), the shear set-up (3 abs, 5 compares/selects, 2 divides
 # + 1 reciprocal, 9 selects = 20), the watertight test on eye-relative
 # vertices (50) and the key (3).
-LPT_VARIANTS = (6, 7)   # render variants in longest-first chunk order (k_render_lp_lpt)
+LPT_VARIANTS = (0, 6, 7)   # render variants in longest-first chunk order (k_render_lp_lpt)
 OPS_PER_PREFILTER = 13
 OPS_PER_PIXEL_TEST = 88
 

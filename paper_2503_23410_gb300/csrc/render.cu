@@ -314,21 +314,34 @@ cudaError_t launch_lpt(const SceneDev& sc, const B& b, cudaStream_t s, int num_s
     return cudaGetLastError();
 }
 
+// Variant 0, what a session has until it is tuned: the longest-first order for
+// a session's LP casts, else the plain order in 64 registers, both with all
+// hit children of a node sorted; and in scenes of up to kPlainTris triangles the
+// plain order in 72 registers with only the nearest child put first (which
+// variant 0 was everywhere).  The 4K cast of the 1.07 M triangle terrain takes
+// 171 us (198 before), its 1440p GT 345 (385), casts of terrains of 7 to 65 K
+// triangles 97 to 142 us (120 to 166).  In small scenes neither pays: the
+// longest-first bookkeeping costs casts of 60 to 90 us 4 to 6 us, and sorting
+// changes soups of 500 to 4,000 triangles by -20 to +10 % from scene to scene.
+constexpr int kPlainTris = 4096;
+
 template <bool GT, class B>
 cudaError_t launch_variant(const SceneDev& sc, const B& b, int variant, cudaStream_t s, int sms) {
     if (b.total_work <= 0) return cudaSuccess;
-    if (is_lpt_variant(variant)) {
-        if (GT) return launch_one<128, 32, 4, 1, 1, GT>(sc, b, s, sms);
-        return variant == kLptVariant ? launch_lpt<128, 0>(sc, b, s, sms) : launch_lpt<128, 0, true, 7>(sc, b, s, sms);
+    if (GT && is_lpt_variant(variant)) variant = 4;
+    if (variant == 0) {
+        if (sc.n_tris <= kPlainTris) return launch_one<128, 32, 4, 1, 1, GT>(sc, b, s, sms);
+        variant = !GT && b.d[0].lpt ? kLptVariantLean : 4;
     }
     // (threads per block, rays per warp fetch, tree width, child order, min blocks/SM)
     switch (variant) {
-        case 0: return launch_one<128, 32, 4, 1, 1, GT>(sc, b, s, sms);
         case 1: return launch_one<256, 32, 4, 0, 1, GT>(sc, b, s, sms);
         case 2: return launch_one<128, 32, 4, 0, 1, GT>(sc, b, s, sms);
         case 3: return launch_one<128, 32, 2, 0, 1, GT>(sc, b, s, sms);
         case 4: return launch_one<128, 32, 4, 0, 8, GT>(sc, b, s, sms);
-        default: return launch_one<128, 32, 4, 1, 8, GT>(sc, b, s, sms);
+        case 5: return launch_one<128, 32, 4, 1, 8, GT>(sc, b, s, sms);
+        case kLptVariant: return launch_lpt<128, 0>(sc, b, s, sms);
+        default: return launch_lpt<128, 0, true, 7>(sc, b, s, sms);
     }
 }
 }  // namespace

@@ -130,14 +130,17 @@ using BigBatch = Batch<VAFR_MAX_BATCH>;
 static_assert(sizeof(BigBatch) + sizeof(SceneDev) <= 32764, "batch too large for kernel params");
 
 // ---- launch interfaces ---------------------------------------------------------
-// Render variants: threads per block, tree width, child order, register cap;
-// variants 6 and 7 are the longest-first LP order (7: the ray regenerated for
-// shading and at most 72 registers, 7 blocks per SM); the GT keeps variant 0's
-// kernel for both.
+// Render variants: 0 the default rule (launch_variant in render.cu); 1-5 threads
+// per block, tree width, child order, register cap; 6 and 7 the longest-first LP
+// order (7: the ray regenerated for shading and at most 72 registers, 7 blocks
+// per SM), whose GT is variant 4's kernel.
 constexpr int kNumRenderVariants = 8;
 constexpr int kLptVariant = 6;
 constexpr int kLptVariantLean = 7;
+// variants that render with a longest-first order in every batch ...
 __host__ __device__ constexpr bool is_lpt_variant(int v) { return v == kLptVariant || v == kLptVariantLean; }
+// ... and those whose single-session LP casts do
+__host__ __device__ constexpr bool has_lpt_kernel(int v) { return v == 0 || is_lpt_variant(v); }
 // Reconstruct variants: column-run tiles (0-3), row tiles (4-7) and the
 // column-run tile with its LP footprint staged in shared memory (8).
 constexpr int kNumReconVariants = 9;
