@@ -824,7 +824,7 @@ int vafr_render_lp_pt(const vafr_scene* scene, vafr_session* s, int32_t eye_mask
         b.total_work += s->n_texels;
         b.d[b.n++] = f;
     }
-    if (!s->d_path) CUDA_TRY(cudaMalloc(&s->d_path, path_scratch_bytes(s->sms)));
+    if (path_uses_pool(b.total_work, max_diffuse) && !s->d_path) CUDA_TRY(cudaMalloc(&s->d_path, path_scratch_bytes(s->sms)));
     CUDA_TRY(launch_path_lp(scene->dev, b, (unsigned long long)seed, max_diffuse, s->d_path, as_stream(stream), s->sms));
     return VAFR_OK;
 }
@@ -1067,7 +1067,7 @@ int vafr_render_full_gt_pt(const vafr_scene* scene, vafr_session* s, int32_t eye
     b.d[0] = f;
     b.n = 1;
     b.total_work = gt_items(f);
-    if (!s->d_path) CUDA_TRY(cudaMalloc(&s->d_path, path_scratch_bytes(s->sms)));
+    if (path_uses_pool(b.total_work, max_diffuse) && !s->d_path) CUDA_TRY(cudaMalloc(&s->d_path, path_scratch_bytes(s->sms)));
     CUDA_TRY(launch_path_gt(scene->dev, b, (unsigned long long)seed, max_diffuse, s->d_path, as_stream(stream), s->sms));
     return VAFR_OK;
 }

@@ -60,13 +60,13 @@ __device__ __forceinline__ float3 face_normal(const SceneDev& sc, const Ray& r, 
 // traversal has 32 rays until the work runs out, and the primary rays of a
 // chunk are still traced together.
 //
-// One path per lane from its first to its last segment left most lanes idle:
+// One path per lane from its first to its last segment leaves most lanes idle:
 // on the 1.07 M triangle terrain 93 % of the paths have a second segment but
 // 25 % a third and 16 % a fourth, and 14 %, 12 % and 7 % a shadow ray there,
-// while each of these steps took a warp as long as the full ones (308, 695,
-// 1,077 and 1,391 us for the LP buffer at 0 to 3 bounces, 10.6 of 32 lanes
-// active).  With the pool: 298, 638, 889 and 1,064 us (15 lanes; the incoherent
-// bounce rays' leaf tests and pushes are what diverges now).
+// while each of these steps takes a warp nearly as long as the full ones (308,
+// 695, 1,077 and 1,391 us for the LP buffer at 0 to 3 bounces, 10.6 of 32 lanes
+// active).  With the pool 1,391 us become 1,048 (15 lanes; the incoherent bounce
+// rays' leaf tests and pushes are what diverges now).
 // The records also hold what the traversal does not need, so it fits 64
 // registers and kPathBlocks blocks per SM (one path per lane: 93 and 5; 6, 7
 // and 8 blocks measured 1,156, 1,148 and 1,110 us, and 1,064 with all four
@@ -88,32 +88,170 @@ struct PathState {
     unsigned mask[kPoolPaths];   // signature: shadow rays lit / cast
 };
 
-// LP texel or display pixel of a work item: its primary ray and random-number
-// key; false when the item is outside the display.
-template <bool GT>
-__device__ __forceinline__ bool path_ray(const FrameDesc& f, long long local, Ray& r, unsigned long long& key,
-                                         int& slot, int& glo, int& ghi, long long& px) {
-    glo = ghi = -1;
-    if (!GT) {
-        slot = lp_ray(f, (int)local, r, glo, ghi);
-        key = (unsigned long long)(slot - (2 * __ldg(f.work + local).y + 1));   // index in column order, no guards
-        return true;
-    }
+// LP texel (slot and the guard slots that copy it) or display pixel of a work
+// item, and its random-number key.
+struct PathPlace {
+    int slot, glo, ghi;
+    long long px;
+    unsigned long long key;
+};
+
+// Display pixel (x, y) of GT work item `local`; false when outside the display.
+__device__ __forceinline__ bool gt_pixel(const FrameDesc& f, long long local, int& x, int& y) {
     const long long tile = local >> 5;
     const int in = (int)(local & 31);
     const int tiles_x = (f.W + 7) >> 3;
-    const int x = (int)(tile % tiles_x) * 8 + (in & 7);
-    const int y = (int)(tile / tiles_x) * 4 + (in >> 3);
-    if (x >= f.W || y >= f.H) return false;
+    x = (int)(tile % tiles_x) * 8 + (in & 7);
+    y = (int)(tile / tiles_x) * 4 + (in >> 3);
+    return x < f.W && y < f.H;
+}
+
+template <bool GT>
+__device__ __forceinline__ PathPlace path_place(const FrameDesc& f, long long local) {
+    PathPlace p{0, -1, -1, 0, 0ull};
+    if (GT) {
+        int x, y;
+        gt_pixel(f, local, x, y);
+        p.px = (long long)y * f.W + x;
+        p.key = (unsigned long long)p.px;
+    } else {
+        const int2 tc = __ldg(f.work + local);
+        const int2 cc = __ldg(&f.col[tc.y]);
+        p.slot = tc.x;
+        p.glo = tc.x - cc.x == cc.y - 1 ? tc.x - cc.y : -1;
+        p.ghi = tc.x == cc.x ? tc.x + cc.y : -1;
+        p.key = (unsigned long long)(tc.x - (2 * tc.y + 1));   // index in column order, no guards
+    }
+    return p;
+}
+
+// Primary ray of a work item; false when it is outside the display.
+template <bool GT>
+__device__ __forceinline__ bool path_ray(const FrameDesc& f, long long local, Ray& r) {
+    if (!GT) {
+        int glo, ghi;
+        lp_ray(f, (int)local, r, glo, ghi);
+        return true;
+    }
+    int x, y;
+    if (!gt_pixel(f, local, x, y)) return false;
     world_ray(f, f.cr * ((float)x + 0.5f - 0.5f * (float)f.W), f.cr * (0.5f * (float)f.H - ((float)y + 0.5f)), r);
-    px = (long long)y * f.W + x;
-    key = (unsigned long long)px;
     return true;
+}
+
+template <bool GT>
+__device__ __forceinline__ void store_path(const FrameDesc& f, const PathPlace& p, float4 v) {
+    if (GT) {
+        store_px(f.disp, p.px, f.disp_fmt, v);
+    } else {
+        store_px(f.lp, p.slot, f.lp_fmt, v);
+        if (p.glo >= 0) store_px(f.lp, p.glo, f.lp_fmt, v);
+        if (p.ghi >= 0) store_px(f.lp, p.ghi, f.lp_fmt, v);
+    }
+}
+
+// Surface point of hit h of ray r, off the surface along the facing normal n.
+__device__ __forceinline__ void leave_surface(const Ray& r, const Hit& h, const float3& n, float o[3]) {
+    const float px = fmaf(h.t, r.dx, r.ox), py = fmaf(h.t, r.dy, r.oy), pz = fmaf(h.t, r.dz, r.oz);
+    const float off = 1e-5f * fmaxf(1.0f, fmaxf(fabsf(px), fmaxf(fabsf(py), fabsf(pz))));
+    o[0] = fmaf(off, n.x, px);
+    o[1] = fmaf(off, n.y, py);
+    o[2] = fmaf(off, n.z, pz);
+}
+
+// Direction of the next segment: cosine-distributed about n.
+__device__ __forceinline__ void bounce(const float3& nn, unsigned long long seed_h, unsigned long long key, int k,
+                                       float d[3]) {
+    const float u1 = pt_uniform(seed_h, key, k, 0), u2 = pt_uniform(seed_h, key, k, 1);
+    float sp, cp;
+    sincospif(2.0f * u2, &sp, &cp);
+    const float rr = sqrtf(u1);
+    const float lx = rr * cp, ly = rr * sp, lz = sqrtf(fmaxf(0.0f, 1.0f - u1));
+    const float sg = copysignf(1.0f, nn.z);
+    const float aa = -1.0f / (sg + nn.z);
+    const float bb = nn.x * nn.y * aa;
+    const float t1x = 1.0f + sg * nn.x * nn.x * aa, t1y = sg * bb, t1z = -sg * nn.x;
+    const float t2x = bb, t2y = sg + nn.y * nn.y * aa, t2z = -nn.y;
+    d[0] = fmaf(lx, t1x, fmaf(ly, t2x, lz * nn.x));
+    d[1] = fmaf(lx, t1y, fmaf(ly, t2y, lz * nn.y));
+    d[2] = fmaf(lx, t1z, fmaf(ly, t2z, lz * nn.z));
 }
 
 // Path signature (LP only): depth + 2 ints per slot: hit id per segment, -1
 // miss, -2 not traced; then the shadow mask: bit k = segment k's shadow ray
 // reached the light, bit 16 + k = it was cast.
+//
+// One path per lane from its first to its last segment: the choice for little
+// work (launch_path_one).
+template <int TPB, int ORDER, bool GT, class B>
+__global__ void __launch_bounds__(TPB)
+k_path_lanes(const SceneDev sc, const __grid_constant__ B b, unsigned long long seed, int depth) {
+    const int lane = threadIdx.x & 31;
+    const unsigned long long seed_h = sm64_mix(seed);
+    const float tlx = -sc.light[0], tly = -sc.light[1], tlz = -sc.light[2];
+    while (true) {
+        unsigned long long base = 0ull;
+        if (lane == 0) base = atomicAdd(b.work_counter, 32ull);
+        base = __shfl_sync(0xffffffffu, base, 0);
+        if ((long long)base >= b.total_work) break;
+        const long long w = (long long)base + lane;
+        if (w >= b.total_work) continue;
+        const FrameDesc& f = b.d[find_frame(b, w, false)];
+        Ray r;
+        if (!path_ray<GT>(f, w - f.work_begin, r)) continue;
+        const PathPlace at = path_place<GT>(f, w - f.work_begin);
+        int* sig = !GT && f.hit_ids ? f.hit_ids + (long long)at.slot * (depth + 2) : nullptr;
+        float beta[3] = {1.0f, 1.0f, 1.0f}, acc[3] = {0.0f, 0.0f, 0.0f};
+        unsigned mask = 0u, fault = 0u;
+        int k = 0;
+        for (; k <= depth; ++k) {
+            ray_setup(r);
+            Hit h;
+            fault |= traverse4<false, ORDER, true>(sc, r, h, nullptr, nullptr, nullptr);
+            if (sig) sig[k] = h.leaf >= 0 ? h.id : -1;
+            if (h.leaf < 0) {
+                const float3 sky = sky_rgb(r.dx, r.dy, r.dz);
+                acc[0] = fmaf(beta[0], sky.x, acc[0]);
+                acc[1] = fmaf(beta[1], sky.y, acc[1]);
+                acc[2] = fmaf(beta[2], sky.z, acc[2]);
+                ++k;
+                break;
+            }
+            const float3 n = face_normal(sc, r, h.leaf);
+            float o[3];
+            leave_surface(r, h, n, o);
+            const float4 rho = __ldg(sc.albedo + h.id);
+            beta[0] *= rho.x; beta[1] *= rho.y; beta[2] *= rho.z;
+            const float cosl = fmaf(n.x, tlx, fmaf(n.y, tly, n.z * tlz));
+            r.ox = o[0]; r.oy = o[1]; r.oz = o[2];
+            r.skip = h.id;
+            if (cosl > 0.0f) {   // a shadow ray is cast
+                mask |= 1u << (16 + k);
+                r.dx = tlx; r.dy = tly; r.dz = tlz;
+                ray_setup(r);
+                Hit hs;
+                fault |= traverse4<false, ORDER, true>(sc, r, hs, nullptr, nullptr, nullptr, true);
+                if (hs.leaf < 0) {
+                    mask |= 1u << k;
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) acc[c] = fmaf(beta[c], cosl, acc[c]);
+                }
+            }
+            if (k < depth) {
+                float d[3];
+                bounce(n, seed_h, at.key, k, d);
+                r.dx = d[0]; r.dy = d[1]; r.dz = d[2];
+            }
+        }
+        if (fault) atomicOr(f.status, fault);
+        store_path<GT>(f, at, make_float4(acc[0], acc[1], acc[2], 1.0f));
+        if (sig) {
+            for (k = min(k, depth + 1); k <= depth; ++k) sig[k] = -2;
+            sig[depth + 1] = (int)mask;
+        }
+    }
+}
+
 template <int TPB, int ORDER, bool GT, int MINB, class B>
 __global__ void __launch_bounds__(TPB, MINB)
 k_path(const SceneDev sc, const __grid_constant__ B b, unsigned long long seed, int depth, PathState* states) {
@@ -134,13 +272,10 @@ k_path(const SceneDev sc, const __grid_constant__ B b, unsigned long long seed, 
             more = (long long)base < b.total_work;
             const long long w = (long long)base + lane;
             Ray r;
-            unsigned long long key;
-            int slot, glo, ghi;
-            long long px;
             bool live = w < b.total_work;
             if (live) {
                 const FrameDesc& f = b.d[find_frame(b, w, false)];
-                live = path_ray<GT>(f, w - f.work_begin, r, key, slot, glo, ghi, px);
+                live = path_ray<GT>(f, w - f.work_begin, r);
             }
             const unsigned lm = __ballot_sync(full, live);
             if (live) {
@@ -156,12 +291,21 @@ k_path(const SceneDev sc, const __grid_constant__ B b, unsigned long long seed, 
             if (count < 32 && more) continue;
         }
         if (count == 0) break;
+        // Once the work has run out and 16 records or fewer are left, a record at
+        // a shadow ray also gets its next segment traced, by lane + 16: the paths
+        // that end the launch take fewer steps.
+        const bool pairs = !more && count <= 16;
         const int n = min(count, 32);
-        const int q = count - n + lane;   // this lane's record
-        const bool on = lane < n;
+        const int idx = pairs ? lane & 15 : lane;
+        const bool second = pairs && lane >= 16;
+        const int q = count - n + idx;   // this lane's record
+        const bool on = idx < n && !second;
         Hit h;
-        if (on) {
-            const bool shadow = P.step[q] & 1u;
+        h.t = INFINITY;
+        h.leaf = -1;
+        h.id = INT_MAX;
+        if (on || (second && idx < n && (P.step[q] & 1u) && (int)(P.step[q] >> 1) < depth)) {
+            const bool shadow = on && (P.step[q] & 1u);
             Ray r;
             r.ox = P.o[0][q]; r.oy = P.o[1][q]; r.oz = P.o[2][q];
             r.dx = shadow ? tlx : P.d[0][q];
@@ -173,6 +317,17 @@ k_path(const SceneDev sc, const __grid_constant__ B b, unsigned long long seed, 
             if (fault) atomicOr(b.d[find_frame(b, (long long)P.work[q], false)].status, fault);
         }
         __syncwarp();
+        Hit next = h;      // closest hit of this lane's record, where it was traced
+        if (pairs) {
+            const int src = idx + 16;
+            const float t2 = __shfl_sync(full, h.t, src);
+            const int leaf2 = __shfl_sync(full, h.leaf, src), id2 = __shfl_sync(full, h.id, src);
+            if (on && (P.step[q] & 1u)) {
+                next.t = t2;
+                next.leaf = leaf2;
+                next.id = id2;
+            }
+        }
         bool go = false;   // the path has another ray
         float o[3], d[3], beta[3] = {1.0f, 1.0f, 1.0f}, acc[3] = {0.0f, 0.0f, 0.0f}, cosl = 0.0f;
         int skip = -1;
@@ -194,58 +349,44 @@ k_path(const SceneDev sc, const __grid_constant__ B b, unsigned long long seed, 
                     acc[c] = __ldcg(&S.acc[c][q]);
                 }
             }
-            const int k = (int)(step >> 1);
+            int k = (int)(step >> 1);
             const FrameDesc& f = b.d[find_frame(b, (long long)work, false)];
-            const long long local = (long long)work - f.work_begin;
-            Ray r;
-            unsigned long long key = 0ull;
-            int slot = 0, glo = -1, ghi = -1;
-            long long px = 0;
-            path_ray<GT>(f, local, r, key, slot, glo, ghi, px);
-            int* sig = !GT && f.hit_ids ? f.hit_ids + (long long)slot * (depth + 2) : nullptr;
-            if (step & 1u) {
+            const PathPlace at = path_place<GT>(f, (long long)work - f.work_begin);
+            int* sig = !GT && f.hit_ids ? f.hit_ids + (long long)at.slot * (depth + 2) : nullptr;
+            bool closest = !(step & 1u);
+            if (!closest) {
                 if (h.leaf < 0) {
                     cosl = __ldcg(&S.cosl[q]);
                     mask |= 1u << k;
 #pragma unroll
                     for (int c = 0; c < 3; ++c) acc[c] = fmaf(beta[c], cosl, acc[c]);
                 }
-                go = k < depth;
-                step = 2u * (unsigned)(k + 1);
-            } else {
-                if (sig) sig[k] = h.leaf >= 0 ? h.id : -1;
-                if (h.leaf < 0) {
+                if (k < depth) {
+                    go = true;
+                    step = 2u * (unsigned)++k;
+                    closest = pairs;
+                }
+            }
+            if (closest) {
+                go = false;
+                if (sig) sig[k] = next.leaf >= 0 ? next.id : -1;
+                if (next.leaf < 0) {
                     const float3 sky = sky_rgb(d[0], d[1], d[2]);
                     acc[0] = fmaf(beta[0], sky.x, acc[0]);
                     acc[1] = fmaf(beta[1], sky.y, acc[1]);
                     acc[2] = fmaf(beta[2], sky.z, acc[2]);
                 } else {
+                    Ray r;
                     r.ox = o[0]; r.oy = o[1]; r.oz = o[2];
                     r.dx = d[0]; r.dy = d[1]; r.dz = d[2];
-                    const float3 nn = face_normal(sc, r, h.leaf);
-                    float pnx = fmaf(h.t, r.dx, r.ox), pny = fmaf(h.t, r.dy, r.oy), pnz = fmaf(h.t, r.dz, r.oz);
-                    const float off = 1e-5f * fmaxf(1.0f, fmaxf(fabsf(pnx), fmaxf(fabsf(pny), fabsf(pnz))));
-                    o[0] = fmaf(off, nn.x, pnx);
-                    o[1] = fmaf(off, nn.y, pny);
-                    o[2] = fmaf(off, nn.z, pnz);
-                    const float4 rho = __ldg(sc.albedo + h.id);
+                    const float3 nn = face_normal(sc, r, next.leaf);
+                    leave_surface(r, next, nn, o);
+                    const float4 rho = __ldg(sc.albedo + next.id);
                     beta[0] *= rho.x; beta[1] *= rho.y; beta[2] *= rho.z;
-                    skip = h.id;
+                    skip = next.id;
                     cosl = fmaf(nn.x, tlx, fmaf(nn.y, tly, nn.z * tlz));
                     if (k < depth) {
-                        const float u1 = pt_uniform(seed_h, key, k, 0), u2 = pt_uniform(seed_h, key, k, 1);
-                        float sp, cp;
-                        sincospif(2.0f * u2, &sp, &cp);
-                        const float rr = sqrtf(u1);
-                        const float lx = rr * cp, ly = rr * sp, lz = sqrtf(fmaxf(0.0f, 1.0f - u1));
-                        const float sg = copysignf(1.0f, nn.z);
-                        const float aa = -1.0f / (sg + nn.z);
-                        const float bb = nn.x * nn.y * aa;
-                        const float t1x = 1.0f + sg * nn.x * nn.x * aa, t1y = sg * bb, t1z = -sg * nn.x;
-                        const float t2x = bb, t2y = sg + nn.y * nn.y * aa, t2z = -nn.y;
-                        d[0] = fmaf(lx, t1x, fmaf(ly, t2x, lz * nn.x));
-                        d[1] = fmaf(lx, t1y, fmaf(ly, t2y, lz * nn.y));
-                        d[2] = fmaf(lx, t1z, fmaf(ly, t2z, lz * nn.z));
+                        bounce(nn, seed_h, at.key, k, d);
                     }
                     if (cosl > 0.0f) {   // a shadow ray is cast
                         mask |= 1u << (16 + k);
@@ -258,17 +399,10 @@ k_path(const SceneDev sc, const __grid_constant__ B b, unsigned long long seed, 
                 }
             }
             if (!go) {
-                const float4 v = make_float4(acc[0], acc[1], acc[2], 1.0f);
-                if (GT) {
-                    store_px(f.disp, px, f.disp_fmt, v);
-                } else {
-                    store_px(f.lp, slot, f.lp_fmt, v);
-                    if (glo >= 0) store_px(f.lp, glo, f.lp_fmt, v);
-                    if (ghi >= 0) store_px(f.lp, ghi, f.lp_fmt, v);
-                    if (sig) {
-                        for (int j = k + 1; j <= depth; ++j) sig[j] = -2;
-                        sig[depth + 1] = (int)mask;
-                    }
+                store_path<GT>(f, at, make_float4(acc[0], acc[1], acc[2], 1.0f));
+                if (sig) {
+                    for (int j = k + 1; j <= depth; ++j) sig[j] = -2;
+                    sig[depth + 1] = (int)mask;
                 }
             }
         }
@@ -300,9 +434,12 @@ cudaError_t launch_path_one(const SceneDev& sc, const B& b, unsigned long long s
                             cudaStream_t s, int num_sms) {
     if (b.total_work <= 0) return cudaSuccess;
     constexpr int TPB = 128;
-    auto kern = k_path<TPB, 0, GT, kPathBlocks, B>;
+    auto pooled = k_path<TPB, 0, GT, kPathBlocks, B>;
+    auto lanes = k_path_lanes<TPB, 1, GT, B>;
+    const bool pool = path_uses_pool(b.total_work, depth);
     int per_sm = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, TPB, 0);
+    cudaError_t e = pool ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pooled, TPB, 0)
+                         : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lanes, TPB, 0);
     if (e != cudaSuccess) return e;
     per_sm = min(max(per_sm, 1), kPathBlocks);   // the scratch holds this many blocks' pools
     e = cudaMemsetAsync(b.work_counter, 0, sizeof(unsigned long long), s);
@@ -310,11 +447,24 @@ cudaError_t launch_path_one(const SceneDev& sc, const B& b, unsigned long long s
     long long grid = (long long)per_sm * num_sms;
     const long long need = (b.total_work + TPB - 1) / TPB;
     if (need < grid) grid = need < 1 ? 1 : need;
-    kern<<<(unsigned)grid, TPB, 0, s>>>(sc, b, seed, depth, static_cast<PathState*>(scratch));
+    if (pool)
+        pooled<<<(unsigned)grid, TPB, 0, s>>>(sc, b, seed, depth, static_cast<PathState*>(scratch));
+    else
+        lanes<<<(unsigned)grid, TPB, 0, s>>>(sc, b, seed, depth);
     count_launch(1);
     return cudaGetLastError();
 }
 }  // namespace
+
+// Gathering the paths pays once enough of them go on: the pool's last paths of
+// each warp take a step at a time with few lanes, some tenths of a launch of
+// one LP buffer.  Measured at 0.7 and 1.06 M texels on terrains of 7 K to 1.07 M
+// triangles, one path per lane against the pool: no bounce 150 against 158 us
+// (the shadow rays keep nine lanes in ten busy anyway), one bounce 287 against
+// 288 and 142 against 146, two 283 against 286 (0.7 M) and 411 against 399
+// (1.06 M), three 352 against 364 (0.7 M) and 528 against 497 (1.06 M); two at
+// 2.07 M pixels 1,440 against 1,139.  So the line lies at 2.5 M bounces.
+bool path_uses_pool(long long work, int depth) { return (long long)depth * work >= 2500000; }
 
 size_t path_scratch_bytes(int num_sms) {
     return sizeof(PathState) * (size_t)num_sms * kPathBlocks * 4;

@@ -1,6 +1,7 @@
-"""The path tracer's pool of waiting paths at its edges: fewer paths than a
-warp, remainders, odd displays, both eyes in one launch, no and many bounces,
-against the FP64 oracle."""
+"""The path tracer at the edges of its work: fewer paths than a warp,
+remainders, odd displays, both eyes in one launch, no and many bounces, on both
+sides of the line between one path per lane and the pool of waiting paths
+(bounces x paths >= 2.5 M), against the FP64 oracle."""
 
 import numpy as np
 import pytest
@@ -58,6 +59,27 @@ def test_small_lp_layouts(V, torch_mod, e_max, depth):
         same = (gsig == rsig).all(1)
         assert (~same).sum() <= _allowed(lay.total, depth)
         assert np.abs(got[same] - ref[same]).max() <= TOL
+    V.vafr_session_destroy(s)
+    V.vafr_scene_destroy(h)
+
+
+@pytest.mark.parametrize("width, height, depth", [(1240, 1000, 2), (1256, 1000, 2), (1781, 707, 2)])
+def test_both_kernels_around_their_line(V, torch_mod, width, height, depth):
+    torch = torch_mod
+    w = workload("random1k")
+    sc, pose = w.scene, w.displays[0].poses[0]
+    h, keep = device_scene(V, sc, torch)
+    s = V.vafr_session_create(V.make_session_desc(width, height, 90.0, [pose]))
+    out = torch.full((height, width, 4), -1.0, dtype=torch.float32, device="cuda")
+    V.vafr_render_full_gt_pt(h, s, 0, out, 9, depth)
+    torch.cuda.synchronize()
+    assert V.vafr_session_check(s) == 0
+    px = np.sort(np.random.default_rng(width).choice(width * height, 20000, replace=False))
+    px = np.unique(np.concatenate([px, np.arange(64), width * height - 1 - np.arange(64)]))
+    o, d = oracle.pixel_rays(width, height, 90.0, pose, px)
+    ref, _ = _oracle_paths(sc, o, d, px, 9, depth)
+    far = np.abs(out.cpu().numpy().reshape(-1, 4)[px] - ref).max(1) > TOL
+    assert far.sum() <= _allowed(len(px), depth)
     V.vafr_session_destroy(s)
     V.vafr_scene_destroy(h)
 
