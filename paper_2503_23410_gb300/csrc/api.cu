@@ -930,7 +930,7 @@ static int deferred_scratch(const vafr_scene* scene_c, cudaStream_t st) {
     if (!rc) rc = scene->alloc(&scene->d_big, n);
     if (!rc) rc = scene->alloc(&scene->d_big_leaf, n);
     if (!rc) rc = scene->alloc(&scene->d_big_first, n);
-    if (!rc) rc = scene->alloc(&scene->d_n_big, 1);
+    if (!rc) rc = scene->alloc(&scene->d_n_big, 2);
     if (rc) return fail(VAFR_ERR_OOM, "deferred scratch");
     CUDA_TRY(launch_leaf_of(scene->dev, scene->d_leaf_of, st, scene->sms));
     return VAFR_OK;

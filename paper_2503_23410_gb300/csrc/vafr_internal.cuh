@@ -191,7 +191,7 @@ struct VbufScratch {
     int4* big;                  // large triangles' pixel boxes
     int* big_leaf;              // ... their leaves
     long long* big_first;       // ... and first tiles
-    unsigned long long* counter;  // (records << 34) | tiles
+    unsigned long long* counter;  // [2]: (records << 34) | tiles; chunks of tiles taken
     unsigned big_cap;
 };
 // stats (device, 4 counters, zeroed by the caller) selects an instrumented
