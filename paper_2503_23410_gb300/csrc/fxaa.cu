@@ -24,11 +24,11 @@
 //             ((3 - 2a) a^2)^2 x 3/4.
 //   7 blend   texel + max(offset, subpix) (neighbour - texel), every channel.
 // Luma and every branch decision use FP32 in one fixed order (no contraction),
-// offsets and the blend FP32.  Two passes, one thread per texel in the
-// frame's screen-space Hilbert order: the luma of every slot into a scratch
-// array, then the filter, which reads lumas (4 bytes) for its neighbourhood
-// and search and colours only for the texel and its blend partner.  The
-// output (a second LP buffer) gets the guard copies too.
+// offsets and the blend FP32.  Two passes: the luma of every slot into a scratch
+// array, then, in the frame's screen-space Hilbert order, the filter, which
+// reads lumas (4 bytes) for its neighbourhood and search and colours only for
+// the texel and its blend partner.  The output (a second LP buffer) gets the
+// guard copies too.
 #include "vafr_internal.cuh"
 
 namespace vafr {
@@ -107,20 +107,36 @@ __device__ __forceinline__ float abs_second_diff(float a, float b, float m) {
     return fabsf(__fsub_rn(__fadd_rn(a, b), __fmul_rn(2.0f, m)));
 }
 
-// The filtered colour of texel (c, j) (slot t, count n).
-__device__ float4 fxaa_texel(const Grid& g, int c, int j, int n, int t) {
+// A texel (c, j) (slot t, count n) with its luma and its neighbours'; the
+// radial neighbours' angular neighbours are the slots beside them.
+struct Cross {
+    int sE, sW;
+    float M, N, S, E, W, range, hi;
+    __device__ __forceinline__ Cross(const Grid& g, int c, int j, const RowDiv& div, int t) {
+        sE = g.at(c, j, div, c + 1, 0);
+        sW = g.at(c, j, div, c - 1, 0);
+        M = g.luma(t);
+        N = g.luma(t + 1);
+        S = g.luma(t - 1);
+        E = g.luma(sE);
+        W = g.luma(sW);
+        const float lo = fminf(M, fminf(fminf(N, S), fminf(E, W)));
+        hi = fmaxf(M, fmaxf(fmaxf(N, S), fmaxf(E, W)));
+        range = __fsub_rn(hi, lo);
+    }
+    // step 1: no edge here
+    __device__ __forceinline__ bool flat() const {
+        return range < fmaxf(1.0f / 12.0f, __fmul_rn(hi, 1.0f / 6.0f));
+    }
+};
+
+// The filtered colour of an edge texel (c, j) (slot t, count n).
+__device__ __forceinline__ float4 fxaa_edge(const Grid& g, int c, int j, int n, int t) {
     const RowDiv div(n);
-    const float M = g.luma(t);
-    // radial neighbours; their angular neighbours are the adjacent slots
-    const int sE = g.at(c, j, div, c + 1, 0), sW = g.at(c, j, div, c - 1, 0);
-    const float N = g.luma(t + 1), S = g.luma(t - 1);
-    const float E = g.luma(sE), W = g.luma(sW);
-    // 1 skip
-    const float lo = fminf(M, fminf(fminf(N, S), fminf(E, W)));
-    const float hi = fmaxf(M, fmaxf(fmaxf(N, S), fmaxf(E, W)));
-    const float range = __fsub_rn(hi, lo);
+    const Cross x(g, c, j, div, t);
+    const int sE = x.sE, sW = x.sW;
+    const float M = x.M, N = x.N, S = x.S, E = x.E, W = x.W, range = x.range;
     const float4 cM = ld_texel(g.lp, g.fmt, t);
-    if (range < fmaxf(1.0f / 12.0f, __fmul_rn(hi, 1.0f / 6.0f))) return cM;
     const float NE = g.luma(sE + 1), SE = g.luma(sE - 1);
     const float NW = g.luma(sW + 1), SW = g.luma(sW - 1);
     // 2 axis
@@ -140,24 +156,34 @@ __device__ float4 fxaa_texel(const Grid& g, int c, int j, int n, int t) {
     // 4 search
     int dist[2];
     float end[2];
+    // along the rows of column c, the partner column's row at the walked texel's
+    // angle is a quotient whose numerator steps by 2 n_partner: it is kept with
+    // its remainder instead of divided for at every step
+    const int cp = min(max(c + side, 0), g.C - 1);
+    const int2 pc = __ldg(g.col + cp);
+    const long long num0 = (long long)(2 * j + 1) * pc.y;
+    const int q0 = cp == c ? j : (pos ? sE : sW) - pc.x;
+    const int rem0 = (int)(num0 - (long long)q0 * (2 * n));   // in [0, 2n)
 #pragma unroll
     for (int d = 0; d < 2; ++d) {
         const int sgn = d ? 1 : -1;
         dist[d] = kFxaaSteps;
         end[d] = 0.0f;
+        int jk = j, q = q0, rem = rem0;
 #pragma unroll 1
         for (int k = 1; k <= kFxaaSteps; ++k) {
             int ta, tb;
             if (across_cols) {   // walk the rows of column c
-                int jk = j + sgn * k;
-                if (n > kFxaaSteps) {            // at most one wrap
-                    jk = jk < 0 ? jk + n : (jk >= n ? jk - n : jk);
-                } else {
-                    jk %= n;
-                    jk = jk < 0 ? jk + n : jk;
+                jk += sgn;
+                rem += sgn * 2 * pc.y;
+                if (jk < 0 || jk == n) {   // the wrap: all of the partner's rows fewer or more
+                    jk -= sgn * n;
+                    q -= sgn * pc.y;
                 }
+                while (rem < 0) { rem += 2 * n; --q; }
+                while (rem >= 2 * n) { rem -= 2 * n; ++q; }
                 ta = cc.x + jk;
-                tb = g.at(c, jk, div, c + side, 0);
+                tb = cp == c ? ta : pc.x + q;
             } else {             // walk the columns at the angle of (c, j)
                 ta = g.at(c, j, div, c + sgn * k, 0);
                 tb = ta + side;
@@ -197,39 +223,78 @@ __device__ __forceinline__ int find_aa_frame(const B& b, long long w) {
     return lo;
 }
 
-// Pass 1: the luma of every texel into the frame's scratch, guard slots too.
+// Pass 1: the luma of every slot into the frame's scratch, in slot order: the
+// thread of the i-th texel takes slot i, and those of the first 2 n_cols also
+// the slots past n_texels (an eye has n_texels + 2 n_cols).
 template <class B>
 __global__ void __launch_bounds__(256) k_lp_luma(const __grid_constant__ B b) {
     for (long long w = (long long)blockIdx.x * 256 + threadIdx.x; w < b.total_aa;
          w += (long long)gridDim.x * 256) {
         const FrameDesc& f = b.d[find_aa_frame(b, w)];
-        const int2 tc = __ldg(f.work + (w - f.aa_begin));   // (slot, column)
-        const int2 cc = __ldg(f.col + tc.y);
-        const int j = tc.x - cc.x, n = cc.y;
-        const float y = luma_of(ld_texel(f.lp, f.lp_fmt, tc.x));
-        f.luma[tc.x] = y;
-        if (j == 0) f.luma[tc.x + n] = y;
-        if (j == n - 1) f.luma[tc.x - n] = y;
+        const int i = (int)(w - f.aa_begin);
+        f.luma[i] = luma_of(ld_texel(f.lp, f.lp_fmt, i));
+        for (int k = i; k < 2 * f.n_cols; k += f.n_texels)
+            f.luma[f.n_texels + k] = luma_of(ld_texel(f.lp, f.lp_fmt, f.n_texels + k));
     }
 }
 
-// Pass 2: the filter.
+// A texel of the batch, and its filtered colour's place (guards included).
+struct AaTexel {
+    const FrameDesc* f;
+    int c, j, n, t;
+    template <class B>
+    __device__ __forceinline__ AaTexel(const B& b, long long w) {
+        f = &b.d[find_aa_frame(b, w)];
+        const int2 tc = __ldg(f->work + (w - f->aa_begin));   // (slot, column)
+        const int2 cc = __ldg(f->col + tc.y);
+        c = tc.y;
+        j = tc.x - cc.x;
+        n = cc.y;
+        t = tc.x;
+    }
+    __device__ __forceinline__ Grid grid() const { return Grid{f->col, f->n_cols, f->lp, f->lp_fmt, f->luma}; }
+    __device__ __forceinline__ void store(float4 v) const {
+        st_texel(f->lp_aa, f->lp_fmt, t, v);
+        if (j == 0) st_texel(f->lp_aa, f->lp_fmt, t + n, v);       // guard after the column
+        if (j == n - 1) st_texel(f->lp_aa, f->lp_fmt, t - n, v);   // guard before it
+    }
+};
+
+// Pass 2: the filter.  A block takes as many texels as it has threads, copies
+// the flat ones and lists the edges, which its first threads then filter side
+// by side.  An LP buffer in FP32 takes 38 us, both passes (47 with 256 threads,
+// each filtering its own texel, a quotient at every step of the search and the
+// lumas in the work order; 40 without the list).  Larger blocks or several
+// texels to a thread lose to the densest blocks, whose searches end the launch.
+constexpr int kFilterThreads = 128;
+
 template <class B>
-__global__ void __launch_bounds__(256, 6) k_fxaa_lp(const __grid_constant__ B b) {
-    for (long long w = (long long)blockIdx.x * 256 + threadIdx.x; w < b.total_aa;
-         w += (long long)gridDim.x * 256) {
-        const FrameDesc& f = b.d[find_aa_frame(b, w)];
-        const int2 tc = __ldg(f.work + (w - f.aa_begin));   // (slot, column)
-        const int2 cc = __ldg(f.col + tc.y);
-        const int j = tc.x - cc.x, n = cc.y;
-        const Grid g{f.col, f.n_cols, f.lp, f.lp_fmt, f.luma};
-        const float4 v = fxaa_texel(g, tc.y, j, n, tc.x);
-        st_texel(f.lp_aa, f.lp_fmt, tc.x, v);
-        if (j == 0) st_texel(f.lp_aa, f.lp_fmt, tc.x + n, v);       // guard after the column
-        if (j == n - 1) st_texel(f.lp_aa, f.lp_fmt, tc.x - n, v);   // guard before it
+__global__ void __launch_bounds__(kFilterThreads, 10) k_fxaa_lp(const __grid_constant__ B b) {
+    __shared__ unsigned short edges[kFilterThreads];
+    __shared__ int n_edges;
+    if (threadIdx.x == 0) n_edges = 0;
+    __syncthreads();
+    const long long w0 = (long long)blockIdx.x * kFilterThreads;
+    const int lane = threadIdx.x & 31;
+    bool edge = false;
+    if (w0 + threadIdx.x < b.total_aa) {
+        const AaTexel x(b, w0 + threadIdx.x);
+        const Grid g = x.grid();
+        const float4 c = ld_texel(g.lp, g.fmt, x.t);
+        edge = !Cross(g, x.c, x.j, RowDiv(x.n), x.t).flat();
+        if (!edge) x.store(c);
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, edge);
+    int at = 0;
+    if (lane == 0 && m) at = atomicAdd(&n_edges, __popc(m));
+    at = __shfl_sync(0xffffffffu, at, 0);
+    if (edge) edges[at + __popc(m & ((1u << lane) - 1u))] = (unsigned short)threadIdx.x;
+    __syncthreads();
+    if ((int)threadIdx.x < n_edges) {
+        const AaTexel x(b, w0 + edges[threadIdx.x]);
+        x.store(fxaa_edge(x.grid(), x.c, x.j, x.n, x.t));
     }
 }
-
 }  // namespace
 
 template <class B>
@@ -239,7 +304,7 @@ cudaError_t launch_fxaa(const B& b, cudaStream_t s, int num_sms) {
     const long long cap = (long long)num_sms * 64;
     const unsigned grid = (unsigned)(want < cap ? want : cap);
     k_lp_luma<B><<<grid, 256, 0, s>>>(b);
-    k_fxaa_lp<B><<<grid, 256, 0, s>>>(b);
+    k_fxaa_lp<B><<<(unsigned)((b.total_aa + kFilterThreads - 1) / kFilterThreads), kFilterThreads, 0, s>>>(b);
     count_launch(2);
     return cudaGetLastError();
 }
