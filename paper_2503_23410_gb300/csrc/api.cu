@@ -275,6 +275,24 @@ cudaError_t lpt_next(LptState* st, unsigned& frames, cudaStream_t s, LptState** 
     return cudaSuccess;
 }
 
+// Scratch of a pooled path tracing launch: the session's, allocated by the first
+// call that wants it.  NULL leaves the launch to the kernel that needs none: for
+// little work, and where the allocation fails.  The relaxed mode keeps it from
+// ending a capture that is under way, on this call's stream or another thread's.
+void* path_scratch(vafr_session* s, long long work, int depth) {
+    if (!path_uses_pool(work, depth)) return nullptr;
+    if (!s->d_path) {
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return nullptr;
+        if (cudaMalloc(&s->d_path, path_scratch_bytes(s->sms)) != cudaSuccess) {
+            cudaGetLastError();
+            s->d_path = nullptr;
+        }
+        cudaThreadExchangeStreamCaptureMode(&mode);
+    }
+    return s->d_path;
+}
+
 int lpt_chunks(int64_t n_texels) { return (int)((n_texels + kLptChunk - 1) / kLptChunk); }
 
 // FP64 per-frame set-up of one eye (Eq. 3): c_r, gaze offsets, gaze split.
@@ -824,8 +842,8 @@ int vafr_render_lp_pt(const vafr_scene* scene, vafr_session* s, int32_t eye_mask
         b.total_work += s->n_texels;
         b.d[b.n++] = f;
     }
-    if (path_uses_pool(b.total_work, max_diffuse) && !s->d_path) CUDA_TRY(cudaMalloc(&s->d_path, path_scratch_bytes(s->sms)));
-    CUDA_TRY(launch_path_lp(scene->dev, b, (unsigned long long)seed, max_diffuse, s->d_path, as_stream(stream), s->sms));
+    void* scratch = path_scratch(s, b.total_work, max_diffuse);
+    CUDA_TRY(launch_path_lp(scene->dev, b, (unsigned long long)seed, max_diffuse, scratch, as_stream(stream), s->sms));
     return VAFR_OK;
 }
 
@@ -1067,8 +1085,8 @@ int vafr_render_full_gt_pt(const vafr_scene* scene, vafr_session* s, int32_t eye
     b.d[0] = f;
     b.n = 1;
     b.total_work = gt_items(f);
-    if (path_uses_pool(b.total_work, max_diffuse) && !s->d_path) CUDA_TRY(cudaMalloc(&s->d_path, path_scratch_bytes(s->sms)));
-    CUDA_TRY(launch_path_gt(scene->dev, b, (unsigned long long)seed, max_diffuse, s->d_path, as_stream(stream), s->sms));
+    void* scratch = path_scratch(s, b.total_work, max_diffuse);
+    CUDA_TRY(launch_path_gt(scene->dev, b, (unsigned long long)seed, max_diffuse, scratch, as_stream(stream), s->sms));
     return VAFR_OK;
 }
 

@@ -436,7 +436,7 @@ cudaError_t launch_path_one(const SceneDev& sc, const B& b, unsigned long long s
     constexpr int TPB = 128;
     auto pooled = k_path<TPB, 0, GT, kPathBlocks, B>;
     auto lanes = k_path_lanes<TPB, 1, GT, B>;
-    const bool pool = path_uses_pool(b.total_work, depth);
+    const bool pool = scratch != nullptr;
     int per_sm = 0;
     cudaError_t e = pool ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pooled, TPB, 0)
                          : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lanes, TPB, 0);

@@ -160,8 +160,8 @@ template <class B>
 cudaError_t launch_reconstruct(const B& batch, int variant, cudaStream_t s);
 // Path-traced LP buffers (pathtrace.cu): one path per texel, `depth` diffuse
 // bounces; FrameDesc.hit_ids, when set, receives depth + 2 ints per slot.
-// Where path_uses_pool says so, `scratch` holds path_scratch_bytes device bytes
-// of the launch's own.
+// `scratch` holds path_scratch_bytes device bytes of the launch's own where
+// path_uses_pool wants the pool, and is NULL for one path per lane.
 bool path_uses_pool(long long work, int depth);
 size_t path_scratch_bytes(int num_sms);
 template <class B>

@@ -125,3 +125,38 @@ def test_odd_displays(V, torch_mod, width, height):
     assert far.sum() <= _allowed(width * height, 2)
     V.vafr_session_destroy(s)
     V.vafr_scene_destroy(h)
+
+
+@pytest.mark.parametrize("depth", [0, 4])
+def test_first_call_inside_a_capture(V, torch_mod, depth):
+    """A session's first path tracing call may be captured: replays give the
+    bits of a direct call, on either side of the line between the kernels."""
+    torch = torch_mod
+    w = workload("random1k")
+    h, keep = device_scene(V, w.scene, torch)
+    bufs = []
+    for captured in (False, True):
+        s = V.vafr_session_create(V.make_session_desc(512, 512, 90.0, w.displays[0].poses))
+        V.vafr_set_gaze(s, 0, 256.0, 256.0)
+        slot, n_slots, _, _ = lp_slots(V, s)
+        lp = torch.full((n_slots, 4), -1.0, dtype=torch.float32, device="cuda")
+        torch.cuda.synchronize()
+        if captured:
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g):
+                V.vafr_render_lp_pt(h, s, 1, lp, 3, depth, None, torch.cuda.current_stream().cuda_stream)
+            assert (lp == -1.0).all()
+            for _ in range(2):
+                lp.fill_(-1.0)
+                g.replay()
+            torch.cuda.synchronize()
+        else:
+            V.vafr_render_lp_pt(h, s, 1, lp, 3, depth)
+        torch.cuda.synchronize()
+        assert V.vafr_session_check(s) == 0
+        bufs.append(lp.cpu().numpy()[slot])
+        if captured:
+            del g
+        V.vafr_session_destroy(s)
+    assert np.array_equal(bufs[0].view(np.int32), bufs[1].view(np.int32))
+    V.vafr_scene_destroy(h)
