@@ -114,6 +114,23 @@ __device__ __forceinline__ float min3f(float a, float b, float c) {
     return d;
 }
 
+// Sort key of a hit child in slot q: its entry distance t >= 0 as bits without
+// the sign (a -0 entry is 0), whose unsigned order is the order of t, with the
+// two low bits replaced by q for an internal child (key word q); a leaf or
+// unused slot has a key word with all but some low bits set and sorts after
+// every distance.  Dropping two bits of t only reorders children whose distances
+// agree within 4 ulp, and a stack entry's distance, rounded down, only culls later.
+__device__ __forceinline__ unsigned child_key(float t, unsigned word) {
+    return (__float_as_uint(t) & 0x7ffffffcu) | word;
+}
+
+// How far from the origin a box may be entered to be visited, for closest hit t:
+// t scaled like a box's far end, finite (a miss is never within it), and with
+// the two low bits set, so that its bits bound the keys of all boxes within it.
+__device__ __forceinline__ float entry_limit(float t) {
+    return __uint_as_float(__float_as_uint(fminf(t * kFarScale, FLT_MAX)) | 3u);
+}
+
 // The four child boxes of a 4-wide node (two pairs of paired-FP32 slabs), with
 // the same robust evaluation as slab2.  Each axis's near and far planes are
 // chosen per ray by the sign of 1/d (the near plane of every box is then its
@@ -121,8 +138,11 @@ __device__ __forceinline__ float min3f(float a, float b, float c) {
 // only the max of three near distances and the min of three far ones.  The
 // node stores each axis as lo, hi, hi, lo: the ray's (near, far) pair is one
 // 256-bit load at a 32-byte offset fixed per ray.
-// Returns the entry distances, +inf for a miss.
-__device__ __forceinline__ float4 slab4(const float4* __restrict__ nd, const Ray& r, float tmax) {
+// A child is hit when it is entered no later than it is left and than `lim`.
+// key: the children's sort keys (child_key; all ones for a miss); hits: bit
+// kHitBit + q for child q.
+__device__ __forceinline__ void slab4(const float4* __restrict__ nd, const Ray& r, float lim, const uint4& word,
+                                      unsigned key[4], unsigned& hits) {
     float4 nxp, fxp, nyp, fyp, nzp, fzp;
     ldg256(nd + r.nx, nxp, fxp);
     ldg256(nd + r.ny, nyp, fyp);
@@ -134,18 +154,19 @@ __device__ __forceinline__ float4 slab4(const float4* __restrict__ nd, const Ray
     const float2 yfa = __fmul2_rn(sub2(fyp.x, fyp.y, r.oy), iy), yfb = __fmul2_rn(sub2(fyp.z, fyp.w, r.oy), iy);
     const float2 zna = __fmul2_rn(sub2(nzp.x, nzp.y, r.oz), iz), znb = __fmul2_rn(sub2(nzp.z, nzp.w, r.oz), iz);
     const float2 zfa = __fmul2_rn(sub2(fzp.x, fzp.y, r.oz), iz), zfb = __fmul2_rn(sub2(fzp.z, fzp.w, r.oz), iz);
-#define VAFR_CHILD(XN, XF, YN, YF, ZN, ZF)                                        \
-    ([&]() {                                                                      \
+    hits = 0u;
+#define VAFR_CHILD(Q, XN, XF, YN, YF, ZN, ZF, W)                                  \
+    {                                                                             \
         const float tn = max3f(XN, YN, fmaxf(ZN, 0.0f));                          \
-        const float tf = min3f(XF, YF, fminf(ZF, tmax));                          \
-        return tn <= tf * kFarScale ? tn : INFINITY;                              \
-    }())
-    const float t0 = VAFR_CHILD(xna.x, xfa.x, yna.x, yfa.x, zna.x, zfa.x);
-    const float t1 = VAFR_CHILD(xna.y, xfa.y, yna.y, yfa.y, zna.y, zfa.y);
-    const float t2 = VAFR_CHILD(xnb.x, xfb.x, ynb.x, yfb.x, znb.x, zfb.x);
-    const float t3 = VAFR_CHILD(xnb.y, xfb.y, ynb.y, yfb.y, znb.y, zfb.y);
+        const bool hit = tn <= fminf(min3f(XF, YF, ZF) * kFarScale, lim);         \
+        key[Q] = hit ? child_key(tn, W) : 0xffffffffu;                            \
+        if (hit) hits |= 1u << (kHitBit + Q);                                     \
+    }
+    VAFR_CHILD(0, xna.x, xfa.x, yna.x, yfa.x, zna.x, zfa.x, word.x)
+    VAFR_CHILD(1, xna.y, xfa.y, yna.y, yfa.y, zna.y, zfa.y, word.y)
+    VAFR_CHILD(2, xnb.x, xfb.x, ynb.x, yfb.x, znb.x, zfb.x, word.z)
+    VAFR_CHILD(3, xnb.y, xfb.y, ynb.y, yfb.y, znb.y, zfb.y, word.w)
 #undef VAFR_CHILD
-    return make_float4(t0, t1, t2, t3);
 }
 
 // Watertight test; returns t or +inf.
@@ -265,18 +286,6 @@ __device__ __forceinline__ void sort2(unsigned& a, unsigned& b) {
     a = lo;
 }
 
-// Sort key of child slot q: its entry distance t >= 0 (+inf for a miss) as
-// bits without the sign (a -0 entry is 0), whose unsigned order is the order
-// of t, with the two low bits replaced by q for an internal child (key word
-// q); a leaf or unused slot has key word all ones and sorts after every miss.
-// Keys below kKeyMiss are hit internal children; dropping two bits of t only
-// reorders children whose distances agree within 4 ulp, and a stack entry's
-// distance, rounded down, only culls later.
-constexpr unsigned kKeyMiss = 0x7f800000u;
-__device__ __forceinline__ unsigned child_key(float t, unsigned word) {
-    return (__float_as_uint(t) & 0x7ffffffcu) | word;
-}
-
 // Closest hit through the 4-wide tree: test the four child boxes, test the
 // leaf children that were hit, then continue with the nearest internal child
 // and push the others far-to-near.  Internal children are ordered by integer
@@ -286,6 +295,14 @@ __device__ __forceinline__ unsigned child_key(float t, unsigned word) {
 // triangle tests per node as its busiest lane needs (not one pass per child
 // slot that any lane needs); the closest-hit rule (t, then id) makes the
 // result independent of the order.
+// The kernels that call this issue on 70 % of the cycles, with the ALU pipe (minima,
+// comparisons, selections, logic) 60 % busy and the FMA pipe 24 %, so what counts
+// is the ALU's work per node: a child's miss is a key of all ones rather than
+// an infinite distance compared again, the leaves come from one mask in the
+// node, and a hit found here drops children through the limit that the keys are
+// compared with anyway.  1.07 M triangles: 4K cast 175 -> 163 us, 1440p GT
+// 345 -> 317; 2 M triangles, both 8K eyes 734 -> 700; 1,024 triangles at 512 x 512
+// 470 -> 430 (frames; the same boxes visited).
 // Returns a fault bit (0 = fine).
 // `any`: an occlusion query, which ends at the first hit found.
 template <bool STATS, int ORDER, bool SKIP = false>
@@ -303,53 +320,38 @@ __device__ __forceinline__ unsigned traverse4(const SceneDev& sc, const Ray& r, 
     unsigned long long stack[kStackSize];
     int sp = 0;
     int node = 0;
+    float lim = entry_limit(INFINITY);
     unsigned budget = 4u * (unsigned)sc.n_tris + 64u;
     while (true) {
         if (--budget == 0u) return kFaultWatchdog;
         if ((unsigned)node >= (unsigned)sc.n_nodes4) return kFaultBadNode;   // the nodes are allocated at their count
         const float4* nd = sc.nodes4 + 16ll * node;
-        float4 t = slab4(nd, r, h.t);
         float4 rf, kwf;
         ldg256(nd + 12, rf, kwf);
         const uint4 kw = make_uint4(__float_as_uint(kwf.x), __float_as_uint(kwf.y), __float_as_uint(kwf.z),
                                     __float_as_uint(kwf.w));
         const int c0 = __float_as_int(rf.x), c1 = __float_as_int(rf.y), c2 = __float_as_int(rf.z),
                   c3 = __float_as_int(rf.w);
+        unsigned key[4], lm;
+        slab4(nd, r, lim, kw, key, lm);
         if (STATS) {
             ++*node_visits;
             *box_tests += (c0 != kEmptyRef) + (c1 != kEmptyRef) + (c2 != kEmptyRef) + (c3 != kEmptyRef);
         }
-        // hit children that are leaves (bit q for child q): references below 0
-        // other than kEmptyRef (INT_MIN: an unused slot with a zero box)
-        static_assert(kEmptyRef == INT_MIN, "the leaf test below relies on kEmptyRef");
-        unsigned lm = 0u;
-#define VAFR_LEAF_BIT(T, C, Q)                                                            \
-        if (T < INFINITY && (unsigned)C > (unsigned)kEmptyRef) lm |= 1u << Q;
-        VAFR_LEAF_BIT(t.x, c0, 0)
-        VAFR_LEAF_BIT(t.y, c1, 1)
-        VAFR_LEAF_BIT(t.z, c2, 2)
-        VAFR_LEAF_BIT(t.w, c3, 3)
-#undef VAFR_LEAF_BIT
-        const float t_entry = h.t;
-        while (lm) {
-            const int q = __ffs(lm) - 1;
-            lm &= lm - 1u;
-            const int C = q == 0 ? c0 : (q == 1 ? c1 : (q == 2 ? c2 : c3));
-            if ((unsigned)~C >= (unsigned)sc.n_tris) return kFaultBadNode;
-            test_leaf<STATS, SKIP>(sc, r, ~C, h, tri_tests);
+        // the hit children that are leaves: slot 3's key word holds the leaves' bits
+        // (none when slot 3 is internal: internal children come first)
+        lm &= kw.w & (15u << kHitBit);
+        if (lm) {
+            do {
+                const int C = lm & (1u << kHitBit) ? c0 : (lm & (2u << kHitBit) ? c1 : (lm & (4u << kHitBit) ? c2 : c3));
+                lm &= lm - 1u;
+                if ((unsigned)~C >= (unsigned)sc.n_tris) return kFaultBadNode;
+                test_leaf<STATS, SKIP>(sc, r, ~C, h, tri_tests);
+            } while (lm);
+            if (any && h.leaf >= 0) return 0u;
+            lim = entry_limit(h.t);   // below it drops the children that start beyond a hit found here
         }
-        if (any && h.leaf >= 0) return 0u;
-        // children entering beyond a closest hit found at this node are dropped
-        // (the box tests already clipped against the hit known before it)
-        if (h.t != t_entry) {
-            const float lim = h.t * kFarScale;
-            if (t.x > lim) t.x = INFINITY;
-            if (t.y > lim) t.y = INFINITY;
-            if (t.z > lim) t.z = INFINITY;
-            if (t.w > lim) t.w = INFINITY;
-        }
-        unsigned k0 = child_key(t.x, kw.x), k1 = child_key(t.y, kw.y), k2 = child_key(t.z, kw.z),
-                 k3 = child_key(t.w, kw.w);
+        unsigned k0 = key[0], k1 = key[1], k2 = key[2], k3 = key[3];
         if (ORDER == 0) {
             // ascending: sorting network (0,1) (2,3) (0,2) (1,3) (1,2)
             sort2(k0, k1);
@@ -363,10 +365,11 @@ __device__ __forceinline__ unsigned traverse4(const SceneDev& sc, const Ray& r, 
             sort2(k2, k3);
             sort2(k0, k2);
         }
-        if (k0 < kKeyMiss) {
+        const unsigned klim = __float_as_uint(lim);
+        if (k0 <= klim) {
             // a stack entry: the child's entry distance (key bits) high, its index low
 #define VAFR_PUSH(K)                                                                      \
-            if (K < kKeyMiss) {                                                           \
+            if (K <= klim) {                                                              \
                 if (sp >= kStackSize) return kFaultStack;                                 \
                 stack[sp++] = ((unsigned long long)(K & ~3u) << 32) | (unsigned)(c0 + (int)(K & 3u)); \
             }
@@ -377,12 +380,11 @@ __device__ __forceinline__ unsigned traverse4(const SceneDev& sc, const Ray& r, 
             node = c0 + (int)(k0 & 3u);
         } else {
             // pop, skipping entries that start beyond the current closest hit
-            const float lim2 = h.t * kFarScale;
             unsigned long long e;
             while (true) {
                 if (sp == 0) return 0u;
                 e = stack[--sp];
-                if (__uint_as_float((unsigned)(e >> 32)) <= lim2) break;
+                if ((unsigned)(e >> 32) <= klim) break;
             }
             node = (int)(unsigned)e;
         }

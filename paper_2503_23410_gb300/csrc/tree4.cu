@@ -605,7 +605,8 @@ __global__ void k_number4(const float4* __restrict__ nodes, const unsigned* __re
 // 4-wide node j from its head: six planes of the four child boxes, the child
 // references (internal 4-wide indices, ~leaf, kEmptyRef for unused slots with
 // a zero box) and the slot keys: q for an internal child in slot q, all ones
-// for the others (the traversal sorts (entry distance | key) as integers).
+// for the others (the traversal sorts (entry distance | key) as integers), but
+// for the bits of slot 3's that tell which slots are leaves.
 // Four lanes to a node: lane q loads child q's box, and the four write the
 // node's rows side by side, 64 bytes at a time (a thread writing all 256 bytes
 // of a node took 63 us for the 343 K nodes of 1.07 M triangles, 41 us so).
@@ -619,7 +620,7 @@ k_pack_nodes4(const float4* __restrict__ nodes, const float* __restrict__ leaf_b
     const bool ok = (unsigned)id < (unsigned)n_inner;   // else past the end, or a malformed binary tree
     float b[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
     int out = kEmptyRef;
-    unsigned key = 0xffffffffu;
+    unsigned key = q == 3 ? kKeyNone3 : 0xffffffffu;
     if (ok) {
         const int i = n_inner - 1 - id;
         int ref[4], m, ni;
@@ -631,6 +632,7 @@ k_pack_nodes4(const float4* __restrict__ nodes, const float* __restrict__ leaf_b
         } else if (q < m) {
             out = r;
         }
+        if (q == 3 && ni < 4) key |= ((1u << m) - (1u << ni)) << kHitBit;
         if (q < m && r >= 0) {
             const float4 l = nodes[2ll * r], h = nodes[2ll * r + 1];
             b[0] = l.x; b[1] = l.y; b[2] = l.z; b[3] = h.x; b[4] = h.y; b[5] = h.z;
