@@ -617,10 +617,10 @@ int vafr_scene_export_tree4(const vafr_scene* scene, int64_t* n_nodes, float* no
                 o[8 * j + 2 * a + 1] = d[4 * a + 1];
             }
             o[8 * j + 6] = d[12];
-            o[8 * j + 7] = d[13];
-            unsigned key3;   // without the leaf slots' bits
-            std::memcpy(&key3, &d[13].w, sizeof(key3));
-            if (key3 != 3u) std::memset(&o[8 * j + 7].w, 0xff, sizeof(key3));
+            unsigned key[4];   // exported: the slot of an internal child, all ones for the others
+            std::memcpy(key, &d[13], sizeof(key));
+            for (unsigned& q : key) q = q >= kInner && q != ~0u ? q & 3u : ~0u;
+            std::memcpy(&o[8 * j + 7], key, sizeof(key));
         }
     }
     if (leaves && n > 0)
@@ -666,18 +666,17 @@ int vafr_scene_inject_fault(vafr_scene* scene, int32_t kind) {
     const int bad = scene->n_nodes4;   // one past the last 4-wide node
     for (int k = 0; k < 4; ++k) {
         const bool used = c[k] != kEmptyRef;
-        if (kind != VAFR_INJECT_NONE && k == 3) q[k] = (int)kKeyNone3;   // no slot is a leaf
         if (kind == VAFR_INJECT_BAD_CHILD && used) {   // every used slot an internal child out of range
             c[k] = bad;
-            q[k] = k;
+            q[k] = (int)(kInner | (unsigned)k);
         }
         if (kind == VAFR_INJECT_LOOP) {   // the root's only child is the root
             c[k] = k == 0 ? 0 : kEmptyRef;
-            if (k < 3) q[k] = k == 0 ? 0 : -1;
+            q[k] = k == 0 ? (int)kInner : -1;
         }
         if (kind == VAFR_INJECT_STACK && used) {   // every used slot leads back to the root
             c[k] = 0;
-            q[k] = 0;
+            q[k] = (int)kInner;
         }
     }
     CUDA_TRY(cudaMemcpy(refs, &v, sizeof(int4), cudaMemcpyHostToDevice));

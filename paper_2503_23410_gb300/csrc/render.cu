@@ -69,7 +69,7 @@ k_render_list(const SceneDev sc, const __grid_constant__ SmallBatch b, const uns
             const int t = lp_ray(f, (int)w, r, glo, ghi);
             ray_setup(r);
             Hit h;
-            const unsigned fault = traverse<4, false, 1>(sc, r, h, nullptr, nullptr, nullptr);
+            const unsigned fault = traverse<4, false>(sc, r, h, nullptr, nullptr, nullptr);
             if (fault) { atomicOr(f.status, fault); h.leaf = -1; h.id = -1; }
             store_lp(f, t, glo, ghi, shade(sc, r, h), h.leaf >= 0 ? h.id : -1);
         }
@@ -318,11 +318,13 @@ cudaError_t launch_lpt(const SceneDev& sc, const B& b, cudaStream_t s, int num_s
 // a session's LP casts, else the plain order in 64 registers, both with all
 // hit children of a node sorted; and in scenes of up to kPlainTris triangles the
 // plain order in 72 registers with only the nearest child put first (which
-// variant 0 was everywhere).  The 4K cast of the 1.07 M triangle terrain takes
-// 171 us (198 before), its 1440p GT 345 (385), casts of terrains of 7 to 65 K
-// triangles 97 to 142 us (120 to 166).  In small scenes neither pays: the
-// longest-first bookkeeping costs casts of 60 to 90 us 4 to 6 us, and sorting
-// changes soups of 500 to 4,000 triangles by -20 to +10 % from scene to scene.
+// variant 0 was everywhere).  Measured against that everywhere: the 4K cast of the
+// 1.07 M triangle terrain 171 us for 198, its 1440p GT 345 for 385, casts of
+// terrains of 7 to 65 K triangles 97 to 142 us for 120 to 166 (since then the
+// traversal takes fewer instructions: 156 and 305 us).  In small scenes neither
+// pays: the longest-first bookkeeping costs casts of 60 to 90 us 4 to 6 us, and
+// sorting changes soups of 500 to 4,000 triangles by -15 to +13 % from scene to
+// scene.
 constexpr int kPlainTris = 4096;
 
 template <bool GT, class B>

@@ -114,21 +114,27 @@ __device__ __forceinline__ float min3f(float a, float b, float c) {
     return d;
 }
 
-// Sort key of a hit child in slot q: its entry distance t >= 0 as bits without
-// the sign (a -0 entry is 0), whose unsigned order is the order of t, with the
-// two low bits replaced by q for an internal child (key word q); a leaf or
-// unused slot has a key word with all but some low bits set and sorts after
-// every distance.  Dropping two bits of t only reorders children whose distances
-// agree within 4 ulp, and a stack entry's distance, rounded down, only culls later.
+// max(a, b, c, 0), NaN if the largest is a NaN: as integers, the non-negative
+// floats keep their order and the negative ones lie below zero.
+__device__ __forceinline__ float max30f(float a, float b, float c) {
+    return __int_as_float(__vimax3_s32_relu(__float_as_int(a), __float_as_int(b), __float_as_int(c)));
+}
+
+// Sort key of a hit child: its entry distance t >= 0 as bits without the sign (a
+// -0 entry is 0), whose unsigned order is the order of t, with the two low bits
+// replaced by the slot q, and the sign bit set for an internal child: leaves sort
+// before internal children.  `word` is the node's: q for a leaf, kInner | q for
+// an internal child, all ones for an unused slot.  Dropping two bits of t only
+// reorders children whose distances agree within 4 ulp, and a stack entry's
+// distance, rounded down, only culls later.
 __device__ __forceinline__ unsigned child_key(float t, unsigned word) {
     return (__float_as_uint(t) & 0x7ffffffcu) | word;
 }
 
-// How far from the origin a box may be entered to be visited, for closest hit t:
-// t scaled like a box's far end, finite (a miss is never within it), and with
-// the two low bits set, so that its bits bound the keys of all boxes within it.
-__device__ __forceinline__ float entry_limit(float t) {
-    return __uint_as_float(__float_as_uint(fminf(t * kFarScale, FLT_MAX)) | 3u);
+// The largest key of an internal child that a ray with closest hit t has to visit:
+// t scaled like a box's far end, and finite (a miss is never within it).
+__device__ __forceinline__ unsigned key_limit(float t) {
+    return __float_as_uint(fminf(t * kFarScale, FLT_MAX)) | kInner | 3u;
 }
 
 // The four child boxes of a 4-wide node (two pairs of paired-FP32 slabs), with
@@ -138,11 +144,11 @@ __device__ __forceinline__ float entry_limit(float t) {
 // only the max of three near distances and the min of three far ones.  The
 // node stores each axis as lo, hi, hi, lo: the ray's (near, far) pair is one
 // 256-bit load at a 32-byte offset fixed per ray.
-// A child is hit when it is entered no later than it is left and than `lim`.
-// key: the children's sort keys (child_key; all ones for a miss); hits: bit
-// kHitBit + q for child q.
-__device__ __forceinline__ void slab4(const float4* __restrict__ nd, const Ray& r, float lim, const uint4& word,
-                                      unsigned key[4], unsigned& hits) {
+// A child is hit when it is entered no later than it is left and, with LIM, than
+// the limit (a key_limit); key: the children's sort keys (child_key), all ones for
+// a miss.
+template <bool LIM>
+__device__ __forceinline__ void slab4(const float4* __restrict__ nd, const Ray& r, const uint4& word, unsigned lim, unsigned key[4]) {
     float4 nxp, fxp, nyp, fyp, nzp, fzp;
     ldg256(nd + r.nx, nxp, fxp);
     ldg256(nd + r.ny, nyp, fyp);
@@ -154,13 +160,13 @@ __device__ __forceinline__ void slab4(const float4* __restrict__ nd, const Ray& 
     const float2 yfa = __fmul2_rn(sub2(fyp.x, fyp.y, r.oy), iy), yfb = __fmul2_rn(sub2(fyp.z, fyp.w, r.oy), iy);
     const float2 zna = __fmul2_rn(sub2(nzp.x, nzp.y, r.oz), iz), znb = __fmul2_rn(sub2(nzp.z, nzp.w, r.oz), iz);
     const float2 zfa = __fmul2_rn(sub2(fzp.x, fzp.y, r.oz), iz), zfb = __fmul2_rn(sub2(fzp.z, fzp.w, r.oz), iz);
-    hits = 0u;
+    const float lf = __uint_as_float(lim & ~kInner);
 #define VAFR_CHILD(Q, XN, XF, YN, YF, ZN, ZF, W)                                  \
     {                                                                             \
-        const float tn = max3f(XN, YN, fmaxf(ZN, 0.0f));                          \
-        const bool hit = tn <= fminf(min3f(XF, YF, ZF) * kFarScale, lim);         \
-        key[Q] = hit ? child_key(tn, W) : 0xffffffffu;                            \
-        if (hit) hits |= 1u << (kHitBit + Q);                                     \
+        const float tn = max30f(XN, YN, ZN);                                      \
+        float tf = min3f(XF, YF, ZF) * kFarScale;                                 \
+        if (LIM) tf = fminf(tf, lf);                                              \
+        key[Q] = tn <= tf ? child_key(tn, W) : ~0u;                               \
     }
     VAFR_CHILD(0, xna.x, xfa.x, yna.x, yfa.x, zna.x, zfa.x, word.x)
     VAFR_CHILD(1, xna.y, xfa.y, yna.y, yfa.y, zna.y, zfa.y, word.y)
@@ -183,7 +189,7 @@ __device__ __forceinline__ float tri_test(const Ray& r, float4 a, float4 b, floa
     const float U = __fsub_rn(__fmul_rn(Cx, By), __fmul_rn(Cy, Bx));
     const float V = __fsub_rn(__fmul_rn(Ax, Cy), __fmul_rn(Ay, Cx));
     const float W = __fsub_rn(__fmul_rn(Bx, Ay), __fmul_rn(By, Ax));
-    if ((U < 0.0f || V < 0.0f || W < 0.0f) && (U > 0.0f || V > 0.0f || W > 0.0f)) return INFINITY;
+    if (min3f(U, V, W) < 0.0f && max3f(U, V, W) > 0.0f) return INFINITY;
     const float det = __fadd_rn(__fadd_rn(U, V), W);
     if (det == 0.0f) return INFINITY;
     const float Az = fmaf(r.mz0, Ax0, fmaf(r.mz1, Ax1, __fmul_rn(r.mz2, Ax2)));
@@ -286,23 +292,50 @@ __device__ __forceinline__ void sort2(unsigned& a, unsigned& b) {
     a = lo;
 }
 
+// The same as signed numbers.
+__device__ __forceinline__ void sort2s(unsigned& a, unsigned& b) {
+    const int lo = min((int)a, (int)b);
+    b = (unsigned)max((int)a, (int)b);
+    a = (unsigned)lo;
+}
+
+// Byte q all ones or zero as the sign bit of argument q.
+__device__ __forceinline__ unsigned signs(unsigned a, unsigned b, unsigned c, unsigned d) {
+    unsigned x, y, z;
+    asm("prmt.b32 %0, %1, %2, 0x00fb;" : "=r"(x) : "r"(a), "r"(b));
+    asm("prmt.b32 %0, %1, %2, 0xfb00;" : "=r"(y) : "r"(c), "r"(d));
+    asm("prmt.b32 %0, %1, %2, 0x7610;" : "=r"(z) : "r"(x), "r"(y));
+    return z;
+}
+
 // Closest hit through the 4-wide tree: test the four child boxes, test the
 // leaf children that were hit, then continue with the nearest internal child
-// and push the others far-to-near.  Internal children are ordered by integer
-// keys (entry distance bits and slot); they are consecutive nodes, so the
-// slot in a key's low bits gives the child's index.  The hit leaf children of
-// a node form a bit mask that one loop consumes, so a warp runs as many
-// triangle tests per node as its busiest lane needs (not one pass per child
-// slot that any lane needs); the closest-hit rule (t, then id) makes the
-// result independent of the order.
+// and push the others far-to-near.  Children are ordered by integer keys (entry
+// distance bits and slot); internal children are consecutive nodes, so the slot
+// in a key's low bits gives the child's index.  One loop takes the hit leaves of
+// a node, so a warp runs as many triangle tests per node as its busiest lane
+// needs (not one pass per child slot that any lane needs); the closest-hit rule
+// (t, then id) makes the result independent of the order.
+//
+// ORDER 0 sorts all four keys.  The leaves come first, so the loop takes the
+// nearest first and passes over those beyond the closest hit, and the box tests
+// need not look at that hit at all.  ORDER 1 only finds the nearest internal child;
+// the box tests drop what lies beyond the closest hit, and the loop takes the
+// leaves from a mask of the keys' signs: shorter chains from a node to its
+// triangles, which small scenes of large overlapping triangles want (their time is
+// that of the longest ray).
+//
 // The kernels that call this issue on 70 % of the cycles, with the ALU pipe (minima,
 // comparisons, selections, logic) 60 % busy and the FMA pipe 24 %, so what counts
-// is the ALU's work per node: a child's miss is a key of all ones rather than
-// an infinite distance compared again, the leaves come from one mask in the
-// node, and a hit found here drops children through the limit that the keys are
-// compared with anyway.  1.07 M triangles: 4K cast 175 -> 163 us, 1440p GT
-// 345 -> 317; 2 M triangles, both 8K eyes 734 -> 700; 1,024 triangles at 512 x 512
-// 470 -> 430 (frames; the same boxes visited).
+// is the ALU's work per node.  A miss is a key of all ones rather than an
+// infinite distance compared again, the closest hit drops internal children
+// through the limit that the keys are compared with anyway, and a stack entry is
+// the key as it is.  With infinite distances and references looked at per child
+// the 4K cast of 1.07 M triangles took 175 us, now 156; 1440p GT 345, now 305; both
+// 8K eyes of 2 M triangles 734, now 680; ORDER 1 on 1,024 triangles at 512 x 512 470,
+// now 426.  Where both orders were measured: terrains of 4,800 to 180,000
+// triangles 105 to 157 us with ORDER 0, 109 to 168 with 1; soups of 1,024 325 to 807
+// with 0, 295 to 760 with 1.
 // Returns a fault bit (0 = fine).
 // `any`: an occlusion query, which ends at the first hit found.
 template <bool STATS, int ORDER, bool SKIP = false>
@@ -320,7 +353,7 @@ __device__ __forceinline__ unsigned traverse4(const SceneDev& sc, const Ray& r, 
     unsigned long long stack[kStackSize];
     int sp = 0;
     int node = 0;
-    float lim = entry_limit(INFINITY);
+    unsigned lim = key_limit(INFINITY);
     unsigned budget = 4u * (unsigned)sc.n_tris + 64u;
     while (true) {
         if (--budget == 0u) return kFaultWatchdog;
@@ -332,26 +365,13 @@ __device__ __forceinline__ unsigned traverse4(const SceneDev& sc, const Ray& r, 
                                     __float_as_uint(kwf.w));
         const int c0 = __float_as_int(rf.x), c1 = __float_as_int(rf.y), c2 = __float_as_int(rf.z),
                   c3 = __float_as_int(rf.w);
-        unsigned key[4], lm;
-        slab4(nd, r, lim, kw, key, lm);
+        unsigned k[4];
+        slab4<ORDER != 0>(nd, r, kw, lim, k);
         if (STATS) {
             ++*node_visits;
             *box_tests += (c0 != kEmptyRef) + (c1 != kEmptyRef) + (c2 != kEmptyRef) + (c3 != kEmptyRef);
         }
-        // the hit children that are leaves: slot 3's key word holds the leaves' bits
-        // (none when slot 3 is internal: internal children come first)
-        lm &= kw.w & (15u << kHitBit);
-        if (lm) {
-            do {
-                const int C = lm & (1u << kHitBit) ? c0 : (lm & (2u << kHitBit) ? c1 : (lm & (4u << kHitBit) ? c2 : c3));
-                lm &= lm - 1u;
-                if ((unsigned)~C >= (unsigned)sc.n_tris) return kFaultBadNode;
-                test_leaf<STATS, SKIP>(sc, r, ~C, h, tri_tests);
-            } while (lm);
-            if (any && h.leaf >= 0) return 0u;
-            lim = entry_limit(h.t);   // below it drops the children that start beyond a hit found here
-        }
-        unsigned k0 = key[0], k1 = key[1], k2 = key[2], k3 = key[3];
+        unsigned k0 = k[0], k1 = k[1], k2 = k[2], k3 = k[3];
         if (ORDER == 0) {
             // ascending: sorting network (0,1) (2,3) (0,2) (1,3) (1,2)
             sort2(k0, k1);
@@ -359,40 +379,63 @@ __device__ __forceinline__ unsigned traverse4(const SceneDev& sc, const Ray& r, 
             sort2(k0, k2);
             sort2(k1, k3);
             sort2(k1, k2);
+            // the leaves, nearest first; what is left are the internal children
+            while (k0 < kInner) {
+                if ((k0 | kInner) <= lim) {
+                    const int C = k0 & 2u ? (k0 & 1u ? c3 : c2) : (k0 & 1u ? c1 : c0);
+                    if ((unsigned)~C >= (unsigned)sc.n_tris) return kFaultBadNode;
+                    test_leaf<STATS, SKIP>(sc, r, ~C, h, tri_tests);
+                    if (any && h.leaf >= 0) return 0u;
+                    lim = key_limit(h.t);
+                }
+                k0 = k1;
+                k1 = k2;
+                k2 = k3;
+                k3 = ~0u;
+            }
         } else {
-            // nearest first, the rest in slot order: (0,1) (2,3) (0,2)
-            sort2(k0, k1);
-            sort2(k2, k3);
-            sort2(k0, k2);
+            unsigned lm = ~signs(k0, k1, k2, k3) & 0x80808080u;
+            if (lm) {
+                do {
+                    const int C = lm & 0x80u ? c0 : (lm & 0x8000u ? c1 : (lm & 0x800000u ? c2 : c3));
+                    lm &= lm - 1u;
+                    if ((unsigned)~C >= (unsigned)sc.n_tris) return kFaultBadNode;
+                    test_leaf<STATS, SKIP>(sc, r, ~C, h, tri_tests);
+                } while (lm);
+                if (any && h.leaf >= 0) return 0u;
+                lim = key_limit(h.t);
+            }
+            sort2s(k0, k1);
+            sort2s(k2, k3);
+            sort2s(k0, k2);
+            // (as signed numbers internal children come first, and misses and leaves are past the limit)
         }
-        const unsigned klim = __float_as_uint(lim);
-        if (k0 <= klim) {
-            // a stack entry: the child's entry distance (key bits) high, its index low
+        unsigned long long e = ((unsigned long long)k0 << 32) | (unsigned)c0;
+#define VAFR_IN(K) (ORDER == 0 ? K <= lim : (int)K <= (int)lim)
+        if (VAFR_IN(k0)) {
+            // a stack entry: the child's key high, its node's first child low
 #define VAFR_PUSH(K)                                                                      \
-            if (K <= klim) {                                                              \
+            if (VAFR_IN(K)) {                                                             \
                 if (sp >= kStackSize) return kFaultStack;                                 \
-                stack[sp++] = ((unsigned long long)(K & ~3u) << 32) | (unsigned)(c0 + (int)(K & 3u)); \
+                stack[sp++] = ((unsigned long long)K << 32) | (unsigned)c0;               \
             }
             VAFR_PUSH(k3)
             VAFR_PUSH(k2)
             VAFR_PUSH(k1)
 #undef VAFR_PUSH
-            node = c0 + (int)(k0 & 3u);
         } else {
             // pop, skipping entries that start beyond the current closest hit
-            unsigned long long e;
-            while (true) {
+            do {
                 if (sp == 0) return 0u;
                 e = stack[--sp];
-                if ((unsigned)(e >> 32) <= klim) break;
-            }
-            node = (int)(unsigned)e;
+            } while ((unsigned)(e >> 32) > lim);
         }
+#undef VAFR_IN
+        node = (int)(unsigned)e + (int)((unsigned)(e >> 32) & 3u);
     }
 }
 
-// WIDE: 4 (4-wide PLOC tree) or 2 (binary LBVH); ORDER (4-wide only): 0 pushes
-// children far-to-near after a full sort, 1 only puts the nearest first.
+// WIDE: 4 (4-wide PLOC tree) or 2 (binary LBVH); ORDER as traverse4's.
 template <int WIDE, bool STATS, int ORDER = 0>
 __device__ __forceinline__ unsigned traverse(const SceneDev& sc, const Ray& r, Hit& h,
                                              unsigned long long* nv, unsigned long long* bt,

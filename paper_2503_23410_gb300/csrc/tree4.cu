@@ -604,9 +604,9 @@ __global__ void k_number4(const float4* __restrict__ nodes, const unsigned* __re
 
 // 4-wide node j from its head: six planes of the four child boxes, the child
 // references (internal 4-wide indices, ~leaf, kEmptyRef for unused slots with
-// a zero box) and the slot keys: q for an internal child in slot q, all ones
-// for the others (the traversal sorts (entry distance | key) as integers), but
-// for the bits of slot 3's that tell which slots are leaves.
+// a zero box) and the slot keys: kInner | q for an internal child in slot q, q
+// for a leaf, all ones for an unused slot (the traversal sorts (entry distance |
+// key) as integers).
 // Four lanes to a node: lane q loads child q's box, and the four write the
 // node's rows side by side, 64 bytes at a time (a thread writing all 256 bytes
 // of a node took 63 us for the 343 K nodes of 1.07 M triangles, 41 us so).
@@ -620,7 +620,7 @@ k_pack_nodes4(const float4* __restrict__ nodes, const float* __restrict__ leaf_b
     const bool ok = (unsigned)id < (unsigned)n_inner;   // else past the end, or a malformed binary tree
     float b[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
     int out = kEmptyRef;
-    unsigned key = q == 3 ? kKeyNone3 : 0xffffffffu;
+    unsigned key = 0xffffffffu;
     if (ok) {
         const int i = n_inner - 1 - id;
         int ref[4], m, ni;
@@ -628,11 +628,11 @@ k_pack_nodes4(const float4* __restrict__ nodes, const float* __restrict__ leaf_b
         const int r = q == 0 ? ref[0] : (q == 1 ? ref[1] : (q == 2 ? ref[2] : ref[3]));
         if (q < ni) {
             out = (int)(1u + sums[i / kHeadThreads] + off[i]) + q;
-            key = (unsigned)q;
+            key = kInner | (unsigned)q;
         } else if (q < m) {
             out = r;
+            key = (unsigned)q;
         }
-        if (q == 3 && ni < 4) key |= ((1u << m) - (1u << ni)) << kHitBit;
         if (q < m && r >= 0) {
             const float4 l = nodes[2ll * r], h = nodes[2ll * r + 1];
             b[0] = l.x; b[1] = l.y; b[2] = l.z; b[3] = h.x; b[4] = h.y; b[5] = h.z;

@@ -19,11 +19,7 @@ enum DeviceFault : unsigned {
 
 constexpr int kStackSize = 128;   // entries; a descent pushes at most 3 per 4-wide level above the last: depth <= 43
 constexpr int kEmptyRef = (int)0x80000000;   // unused slot of a 4-wide node
-// Slot 3's key word in a 4-wide node whose slot 3 is not internal, but for bits
-// kHitBit + q, set where slot q is a leaf.  (A node whose slot 3 is internal has
-// four internal children; its key word, 3, has none of these bits.)
-constexpr int kHitBit = 4;
-constexpr unsigned kKeyNone3 = ~(15u << kHitBit);
+constexpr unsigned kInner = 0x80000000u;     // key word of an internal child in slot q: kInner | q; of a leaf: q
 constexpr int kMaxSeg = VAFR_MAX_PIVOTS - 1;
 
 // ---- scene (LBVH) in traversal layout ----------------------------------------
