@@ -304,7 +304,8 @@ cudaError_t launch_lpt(const SceneDev& sc, const B& b, cudaStream_t s, int num_s
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, TPB, 0);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
-    e = cudaMemsetAsync(b.work_counter, 0, 2 * sizeof(unsigned long long), s);
+    // a frame with an order comes with its state's work counters, cleared with it
+    if (!b.d[0].lpt) e = cudaMemsetAsync(b.work_counter, 0, 2 * sizeof(unsigned long long), s);
     if (e != cudaSuccess) return e;
     long long grid = (long long)per_sm * num_sms;
     const long long need = (b.total_work + TPB - 1) / TPB;

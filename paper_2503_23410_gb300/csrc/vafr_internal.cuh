@@ -66,12 +66,16 @@ constexpr int kUTable = 2048;
 // so the results are those of the plain order.  Without it the slowest chunks,
 // wherever they fall in the work order, decide when the launch ends.  The
 // state has two halves used alternately (frame parity): the half being read
-// holds this frame's list, the other collects the next frame's; the host
-// clears the collecting half's counters before each frame.
+// holds this frame's list, the other collects the next frame's and, in its
+// first frame's state, counts the launch's work; the host clears the collecting
+// half's counters before each frame.
 struct LptCounters {
     unsigned long long cyc_sum;   // sum of the chunk costs of the frame
     unsigned chunks_done;         // chunks costed
     unsigned hot_count;           // entries of the list
+    // work counters of the frame's launch, on a line of their own (next to the others,
+    // whose line every listed chunk updates, a 156 us cast takes 161; so, 154)
+    alignas(128) unsigned long long work[2];
 };
 struct LptState {
     LptCounters ctr[2];
