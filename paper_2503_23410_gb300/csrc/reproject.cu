@@ -60,6 +60,10 @@ __device__ __forceinline__ void st_rgba(void* lp, int fmt, int slot, float4 v) {
     }
 }
 
+// Texels in column order without the guard slots: the compact index of a slot of
+// column c is slot - guards(c).
+__device__ __forceinline__ int guards(int c) { return 2 * c + 1; }
+
 // camera direction of LP work item k of frame f (the render kernel's ray)
 __device__ __forceinline__ void lp_dir(const FrameDesc& f, int k, int& slot, int& col, float3& o, float3& d) {
     const int2 tc = __ldg(f.work + k);
@@ -108,30 +112,34 @@ __global__ void __launch_bounds__(256) k_rep_vertices(const __grid_constant__ Sm
             v.x = piece_eval(__ldg(R.u_tab + i), s - (float)i);
             v.y = angle_fraction(qy, qx, fmaxf(fabsf(qx), 1e-30f));
             v.z = inf ? 1e30f : sqrtf(fmaf(P.x, P.x, fmaf(P.y, P.y, P.z * P.z)));
-            v.w = __int_as_float(1 | (inf ? 2 : 0));
+            v.w = __int_as_float(1 | (inf ? 2 : 0) | col << 2);
         }
-        vert[slot] = v;
+        vert[slot - guards(col)] = v;
     }
 }
 
-// The three left slots of triangle s of left texel (c, j) (see the mesh rule).
-__device__ __forceinline__ bool rep_triangle(const int2* colt, int C, int c, int j, int s, int tv[3]) {
-    const int c2 = s == 0 ? c + 1 : c - 1;
+// The compact indices of the three left texels of triangle s of left texel (c, j),
+// and the column of the third (see the mesh rule).  Rings below 32,768 texels keep
+// the products within 32 bits, and k, at most 3/2 ring sizes, needs one correction
+// and no remainder (the raster pass takes 38 us, with 64-bit divisions and
+// remainders 42).
+__device__ __forceinline__ bool rep_triangle(const int2* colt, int C, int c, int j, int s, int tv[3], int& c2) {
+    c2 = s == 0 ? c + 1 : c - 1;
     if (c2 < 0 || c2 >= C) return false;
     const int2 a = __ldg(colt + c), b = __ldg(colt + c2);
-    const long long n = a.y, n2 = b.y;
     long long k;
-    if (s == 0) {
-        const long long w = ((2ll * j + 3) * n2 + n - 1) / n - 2;
-        k = w >= 0 ? w / 2 : -1;
+    if ((a.y | b.y) < 32768) {
+        const unsigned n = (unsigned)a.y, num = (2u * (unsigned)j + 3u) * (unsigned)b.y;
+        k = s == 0 ? ((int)((num + n - 1u) / n) - 2) >> 1 : ((int)(num / n) - 1) >> 1;
     } else {
-        const long long q = ((2ll * j + 3) * n2) / n;
-        k = q >= 1 ? (q - 1) / 2 : -1;
+        const long long n = a.y, num = (2ll * j + 3) * b.y;
+        k = s == 0 ? ((num + n - 1) / n - 2) >> 1 : (num / n - 1) >> 1;
     }
-    k = ((k % n2) + n2) % n2;
-    tv[0] = a.x + j;
-    tv[1] = a.x + (j + 1 == a.y ? 0 : j + 1);
-    tv[2] = b.x + (int)k;
+    if (k < 0) k += b.y;
+    else if (k >= b.y) k -= b.y;
+    tv[0] = a.x - guards(c) + j;
+    tv[1] = a.x - guards(c) + (j + 1 == a.y ? 0 : j + 1);
+    tv[2] = b.x - guards(c2) + (int)k;
     return true;
 }
 
@@ -178,7 +186,9 @@ __device__ __forceinline__ bool load_tri(const float4* vert, const int tv[3], fl
     return fhi - flo <= kMaxFSpan;
 }
 
-// Pass 2: rasterise the two triangles of every left texel into the z-buffer.
+// Pass 2: rasterise the two triangles of every left texel into the z-buffer: 370
+// instructions to a texel, bound by their latency (58 % of the issue slots at 44 %
+// occupancy; with 48 registers they spill, 6 us slower).
 __global__ void __launch_bounds__(256)
 k_rep_raster(const __grid_constant__ SmallBatch b, const float4* vert, unsigned long long* zbuf) {
     const FrameDesc& L = b.d[0];
@@ -187,10 +197,10 @@ k_rep_raster(const __grid_constant__ SmallBatch b, const float4* vert, unsigned 
     for (int k = blockIdx.x * 256 + threadIdx.x; k < L.n_texels; k += gridDim.x * 256) {
         const int2 tc = __ldg(L.work + k);
         const int c = tc.y, j = tc.x - __ldg(L.col + c).x;
-        const int compact = tc.x - (2 * c + 1);
+        const int compact = tc.x - guards(c);
         for (int s = 0; s < 2; ++s) {
-            int tv[3];
-            if (!rep_triangle(L.col, C, c, j, s, tv)) continue;
+            int tv[3], c2;
+            if (!rep_triangle(L.col, C, c, j, s, tv, c2)) continue;
             float U[3], F[3], Z[3];
             int copies;
             if (!load_tri(vert, tv, U, F, Z, copies)) continue;
@@ -235,12 +245,17 @@ k_rep_raster(const __grid_constant__ SmallBatch b, const float4* vert, unsigned 
 }
 
 // Pass 3: colours of covered right texels, the rest listed as holes.  A
-// block takes 1,024 consecutive work items (4 per thread, in the LP work
+// block takes 512 consecutive work items (2 per thread, in the LP work
 // order) and appends its holes as one contiguous run in that order, so the
 // warps of the hole cast get spatially coherent rays.
-constexpr int kResolveItems = 4;
+// What bounds it is the chain of loads from a texel's key to its colours (vertex,
+// rings, vertices, texels).  The left column comes with the triangle's first vertex;
+// found by a binary search over the columns the pass took 40 us for 1.06 M texels,
+// then 33.  1,024 items a block (1,037 blocks of 56 registers, 1.7 waves) took 5 us
+// more than 512.
+constexpr int kResolveItems = 2;
 
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 5)
 k_rep_resolve(const __grid_constant__ SmallBatch b, const float4* vert, const unsigned long long* zbuf,
               int2* holes, unsigned* count, int* tri_out) {
     const FrameDesc& L = b.d[0];
@@ -270,14 +285,9 @@ k_rep_resolve(const __grid_constant__ SmallBatch b, const float4* vert, const un
             }
             const unsigned tid = (unsigned)(key & 0xffffffffu);
             const int compact = (int)(tid >> 1), sd = (int)(tid & 1u);
-            int lo = 0, hi = C - 1;   // left column holding compact texel `compact`
-            while (lo < hi) {
-                const int mid = (lo + hi + 1) >> 1;
-                if (__ldg(L.col + mid).x - (2 * mid + 1) <= compact) lo = mid; else hi = mid - 1;
-            }
-            const int jl = compact - (__ldg(L.col + lo).x - (2 * lo + 1));
-            int tv[3];
-            rep_triangle(L.col, C, lo, jl, sd, tv);
+            const int cl = __float_as_int(vert[compact].w) >> 2;   // a drawn triangle's vertices have their columns
+            int tv[3], c2;
+            rep_triangle(L.col, C, cl, compact - (__ldg(L.col + cl).x - guards(cl)), sd, tv, c2);
             float U[3], F[3], Z[3];
             int copies;
             load_tri(vert, tv, U, F, Z, copies);
@@ -285,9 +295,9 @@ k_rep_resolve(const __grid_constant__ SmallBatch b, const float4* vert, const un
             const float f = ((float)jr + 0.5f) / (float)rc.y;
             if (!bary(U, F, (float)tc.y, f, w) || fminf(w[0], fminf(w[1], w[2])) < -0.25f)
                 bary(U, F, (float)tc.y, f + 1.0f, w);
-            const float4 a = ld_rgba(L.lp, L.lp_fmt, tv[0]);
-            const float4 bb = ld_rgba(L.lp, L.lp_fmt, tv[1]);
-            const float4 cc = ld_rgba(L.lp, L.lp_fmt, tv[2]);
+            const float4 a = ld_rgba(L.lp, L.lp_fmt, tv[0] + guards(cl));
+            const float4 bb = ld_rgba(L.lp, L.lp_fmt, tv[1] + guards(cl));
+            const float4 cc = ld_rgba(L.lp, L.lp_fmt, tv[2] + guards(c2));
             const float4 v = make_float4(fmaf(w[0], a.x, fmaf(w[1], bb.x, w[2] * cc.x)),
                                          fmaf(w[0], a.y, fmaf(w[1], bb.y, w[2] * cc.y)),
                                          fmaf(w[0], a.z, fmaf(w[1], bb.z, w[2] * cc.z)),
@@ -334,7 +344,7 @@ cudaError_t launch_reproject(const SmallBatch& b, const RepScratch& r, cudaStrea
     if ((e = cudaMemsetAsync(r.count, 0, sizeof(unsigned), s)) != cudaSuccess) return e;
     const unsigned grid = (unsigned)min((b.d[0].n_texels + 255) / 256, num_sms * 16);
     const unsigned rgrid =
-        (unsigned)max(1, min((R.n_texels + 256 * kResolveItems - 1) / (256 * kResolveItems), num_sms * 8));
+        (unsigned)max(1, min((R.n_texels + 256 * kResolveItems - 1) / (256 * kResolveItems), num_sms * 64));
     k_rep_vertices<<<grid, 256, 0, s>>>(b, r.vert);
     k_rep_raster<<<grid, 256, 0, s>>>(b, r.vert, r.zbuf);
     k_rep_resolve<<<rgrid, 256, 0, s>>>(b, r.vert, r.zbuf, r.holes, r.count, r.tri_out);

@@ -182,7 +182,7 @@ cudaError_t launch_render_list(const SceneDev& scene, const SmallBatch& batch, c
 // VaFR_Rep reprojection (reproject.cu): left frame d[0] (lp, depth) warped into
 // right frame d[1] (lp written, holes appended to `holes` / `count`).
 struct RepScratch {
-    float4* vert;                 // [left slots] (U, F, depth, flags) seen from the right eye
+    float4* vert;                 // [left texels] (U, F, depth, flags | column) seen from the right eye
     unsigned long long* zbuf;     // [right slots] (depth bits << 32) | triangle id
     int2* holes;                  // [right texels] (slot, column) left uncovered
     unsigned* count;              // number of holes
