@@ -891,7 +891,7 @@ int vafr_reproject_lp(vafr_session* s, const void* left_lp, const float* left_de
     b.d[1] = s->fd[1];
     b.d[1].lp = right_lp_out;
     b.n = 2;
-    RepScratch r{s->d_rep_vert, s->d_rep_zbuf, s->d_rep_holes, s->d_rep_count, right_tri_out};
+    RepScratch r{s->d_rep_vert, s->d_rep_zbuf, s->d_rep_holes, s->d_rep_count, right_tri_out, nullptr};
     CUDA_TRY(launch_reproject(b, r, as_stream(stream), s->sms));
     return VAFR_OK;
 }
@@ -921,7 +921,7 @@ int vafr_render_lp_rep(const vafr_scene* scene, vafr_session* s, void* lp_out, i
     w.d[1] = s->fd[1];
     w.d[1].lp = right;
     w.n = 2;
-    RepScratch r{s->d_rep_vert, s->d_rep_zbuf, s->d_rep_holes, s->d_rep_count, right_tri_out};
+    RepScratch r{s->d_rep_vert, s->d_rep_zbuf, s->d_rep_holes, s->d_rep_count, right_tri_out, s->d_counter};
     CUDA_TRY(launch_reproject(w, r, st, s->sms));
     // 3. cast the right eye's holes
     SmallBatch h{};

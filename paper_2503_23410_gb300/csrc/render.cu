@@ -371,8 +371,6 @@ cudaError_t launch_render_list(const SceneDev& scene, const SmallBatch& batch, c
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_render_list, 128, 0);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
-    e = cudaMemsetAsync(batch.work_counter, 0, sizeof(unsigned long long), s);
-    if (e != cudaSuccess) return e;
     k_render_list<<<(unsigned)(per_sm * num_sms), 128, 0, s>>>(scene, batch, count);
     count_launch(1);
     return cudaGetLastError();

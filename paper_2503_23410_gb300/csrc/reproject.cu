@@ -81,10 +81,19 @@ __device__ __forceinline__ void lp_dir(const FrameDesc& f, int k, int& slot, int
     col = tc.y;
 }
 
-// Pass 1: the right-eye (U, F, depth, flags) of every left texel.
-__global__ void __launch_bounds__(256) k_rep_vertices(const __grid_constant__ SmallBatch b, float4* vert) {
+// Pass 1: the right-eye (U, F, depth, flags) of every left texel.  It also clears
+// the z-buffer and the counters that the next passes use (on their own, three
+// launches more).
+__global__ void __launch_bounds__(256) k_rep_vertices(const __grid_constant__ SmallBatch b, const RepScratch r) {
     const FrameDesc& L = b.d[0];
     const FrameDesc& R = b.d[1];
+    float4* const vert = r.vert;
+    const int slots = R.n_texels + guards(R.n_cols) - 1;
+    for (int k = blockIdx.x * 256 + threadIdx.x; k < slots; k += gridDim.x * 256) r.zbuf[k] = kEmptyKey;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        *r.count = 0u;
+        if (r.work) *r.work = 0ull;
+    }
     for (int k = blockIdx.x * 256 + threadIdx.x; k < L.n_texels; k += gridDim.x * 256) {
         int slot, col;
         float3 o, d;
@@ -339,13 +348,10 @@ k_rep_resolve(const __grid_constant__ SmallBatch b, const float4* vert, const un
 
 cudaError_t launch_reproject(const SmallBatch& b, const RepScratch& r, cudaStream_t s, int num_sms) {
     const FrameDesc& R = b.d[1];
-    cudaError_t e = cudaMemsetAsync(r.zbuf, 0xff, sizeof(unsigned long long) * (size_t)(R.n_texels + 2 * R.n_cols), s);
-    if (e != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(r.count, 0, sizeof(unsigned), s)) != cudaSuccess) return e;
     const unsigned grid = (unsigned)min((b.d[0].n_texels + 255) / 256, num_sms * 16);
     const unsigned rgrid =
         (unsigned)max(1, min((R.n_texels + 256 * kResolveItems - 1) / (256 * kResolveItems), num_sms * 64));
-    k_rep_vertices<<<grid, 256, 0, s>>>(b, r.vert);
+    k_rep_vertices<<<grid, 256, 0, s>>>(b, r);
     k_rep_raster<<<grid, 256, 0, s>>>(b, r.vert, r.zbuf);
     k_rep_resolve<<<rgrid, 256, 0, s>>>(b, r.vert, r.zbuf, r.holes, r.count, r.tri_out);
     count_launch(3);

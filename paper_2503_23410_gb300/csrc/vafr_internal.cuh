@@ -176,7 +176,8 @@ template <class B>
 cudaError_t launch_path_gt(const SceneDev& scene, const B& batch, unsigned long long seed, int depth,
                            void* scratch, cudaStream_t s, int num_sms);
 // Ray casting of an explicit list of (slot, column) work items whose count
-// is read from device memory (render.cu): the reprojection's holes.
+// is read from device memory (render.cu): the reprojection's holes.  The batch's
+// work counter has been cleared.
 cudaError_t launch_render_list(const SceneDev& scene, const SmallBatch& batch, const unsigned* count,
                                cudaStream_t s, int num_sms);
 // VaFR_Rep reprojection (reproject.cu): left frame d[0] (lp, depth) warped into
@@ -187,6 +188,7 @@ struct RepScratch {
     int2* holes;                  // [right texels] (slot, column) left uncovered
     unsigned* count;              // number of holes
     int* tri_out;                 // [right slots] winning triangle id / -1, or nullptr
+    unsigned long long* work;     // work counter to clear for the hole cast, or nullptr
 };
 cudaError_t launch_reproject(const SmallBatch& batch, const RepScratch& r, cudaStream_t s, int num_sms);
 // Deferred path (raster.cu): visibility buffer of frame d[0] at display
