@@ -100,53 +100,6 @@ __device__ __forceinline__ bool tri_bbox(const FrameDesc& f, float3 p[3], int& x
     return true;
 }
 
-// The shear set-up of ray_setup alone (the triangle test needs no box data).
-__device__ __forceinline__ void ray_setup_tri(Ray& r) {
-    const float ax = fabsf(r.dx), ay = fabsf(r.dy), az = fabsf(r.dz);
-    const int kz = (ax >= ay && ax >= az) ? 0 : (ay >= az ? 1 : 2);
-    int kx = kz == 2 ? 0 : kz + 1;
-    int ky = kx == 2 ? 0 : kx + 1;
-    const float dkz = kz == 0 ? r.dx : (kz == 1 ? r.dy : r.dz);
-    if (dkz < 0.0f) { const int s = kx; kx = ky; ky = s; }
-    const float dkx = kx == 0 ? r.dx : (kx == 1 ? r.dy : r.dz);
-    const float dky = ky == 0 ? r.dx : (ky == 1 ? r.dy : r.dz);
-    const float Sx = dkx / dkz, Sy = dky / dkz, Sz = 1.0f / dkz;
-    r.mx0 = kx == 0 ? 1.0f : (kz == 0 ? -Sx : 0.0f);
-    r.mx1 = kx == 1 ? 1.0f : (kz == 1 ? -Sx : 0.0f);
-    r.mx2 = kx == 2 ? 1.0f : (kz == 2 ? -Sx : 0.0f);
-    r.my0 = ky == 0 ? 1.0f : (kz == 0 ? -Sy : 0.0f);
-    r.my1 = ky == 1 ? 1.0f : (kz == 1 ? -Sy : 0.0f);
-    r.my2 = ky == 2 ? 1.0f : (kz == 2 ? -Sy : 0.0f);
-    r.mz0 = kz == 0 ? Sz : 0.0f;
-    r.mz1 = kz == 1 ? Sz : 0.0f;
-    r.mz2 = kz == 2 ? Sz : 0.0f;
-}
-
-// The watertight test of trace.cuh's tri_test with the three vertex-minus-
-// origin differences already formed (every pixel ray of a frame starts at the
-// eye, so they are per triangle): the same FP32 operations in the same order,
-// hence the same t bit for bit.
-__device__ __forceinline__ float tri_test_rel(const Ray& r, float3 A, float3 B, float3 C) {
-    const float Ax = fmaf(r.mx0, A.x, fmaf(r.mx1, A.y, __fmul_rn(r.mx2, A.z)));
-    const float Ay = fmaf(r.my0, A.x, fmaf(r.my1, A.y, __fmul_rn(r.my2, A.z)));
-    const float Bx = fmaf(r.mx0, B.x, fmaf(r.mx1, B.y, __fmul_rn(r.mx2, B.z)));
-    const float By = fmaf(r.my0, B.x, fmaf(r.my1, B.y, __fmul_rn(r.my2, B.z)));
-    const float Cx = fmaf(r.mx0, C.x, fmaf(r.mx1, C.y, __fmul_rn(r.mx2, C.z)));
-    const float Cy = fmaf(r.my0, C.x, fmaf(r.my1, C.y, __fmul_rn(r.my2, C.z)));
-    const float U = __fsub_rn(__fmul_rn(Cx, By), __fmul_rn(Cy, Bx));
-    const float V = __fsub_rn(__fmul_rn(Ax, Cy), __fmul_rn(Ay, Cx));
-    const float W = __fsub_rn(__fmul_rn(Bx, Ay), __fmul_rn(By, Ax));
-    if ((U < 0.0f || V < 0.0f || W < 0.0f) && (U > 0.0f || V > 0.0f || W > 0.0f)) return INFINITY;
-    const float det = __fadd_rn(__fadd_rn(U, V), W);
-    if (det == 0.0f) return INFINITY;
-    const float Az = fmaf(r.mz0, A.x, fmaf(r.mz1, A.y, __fmul_rn(r.mz2, A.z)));
-    const float Bz = fmaf(r.mz0, B.x, fmaf(r.mz1, B.y, __fmul_rn(r.mz2, B.z)));
-    const float Cz = fmaf(r.mz0, C.x, fmaf(r.mz1, C.y, __fmul_rn(r.mz2, C.z)));
-    const float T = fmaf(U, Az, fmaf(V, Bz, __fmul_rn(W, Cz)));
-    const float t = __fdiv_rn(T, det);
-    return t > 0.0f ? t : INFINITY;
-}
-
 // Per-triangle raster set-up: world vertices, id, the camera-depth lower
 // bound t_lo of any hit (rays are (cx, cy, 1) in camera space, so a hit's
 // distance t is its camera depth), and the screen-space pre-filter.
@@ -283,7 +236,7 @@ __device__ __forceinline__ void test_queued(const FrameDesc& f, unsigned long lo
         if (STATS) ++c.tests;
         Ray r;
         pixel_ray(f, x, y, r);
-        ray_setup_tri(r);
+        ray_shear(r);   // the triangle test needs no box data
         const float t = tri_test_rel(r, make_float3(A.x, A.y, A.z), make_float3(B.x, B.y, B.z),
                                      make_float3(C.x, C.y, C.z));
         if (t < INFINITY) {
