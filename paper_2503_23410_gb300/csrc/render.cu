@@ -315,19 +315,6 @@ cudaError_t launch_lpt(const SceneDev& sc, const B& b, cudaStream_t s, int num_s
     return cudaGetLastError();
 }
 
-// Variant 0, what a session has until it is tuned: the longest-first order for
-// a session's LP casts, else the plain order in 64 registers, both with all
-// hit children of a node sorted; and in scenes of up to kPlainTris triangles the
-// plain order in 72 registers with only the nearest child put first (which
-// variant 0 was everywhere).  Measured against that everywhere: the 4K cast of the
-// 1.07 M triangle terrain 171 us for 198, its 1440p GT 345 for 385, casts of
-// terrains of 7 to 65 K triangles 97 to 142 us for 120 to 166 (since then the
-// traversal takes fewer instructions: 156 and 305 us).  In small scenes neither
-// pays: the longest-first bookkeeping costs casts of 60 to 90 us 4 to 6 us, and
-// sorting changes soups of 500 to 4,000 triangles by -15 to +13 % from scene to
-// scene.
-constexpr int kPlainTris = 4096;
-
 template <bool GT, class B>
 cudaError_t launch_variant(const SceneDev& sc, const B& b, int variant, cudaStream_t s, int sms) {
     if (b.total_work <= 0) return cudaSuccess;

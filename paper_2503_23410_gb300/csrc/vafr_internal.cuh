@@ -135,17 +135,31 @@ using BigBatch = Batch<VAFR_MAX_BATCH>;
 static_assert(sizeof(BigBatch) + sizeof(SceneDev) <= 32764, "batch too large for kernel params");
 
 // ---- launch interfaces ---------------------------------------------------------
-// Render variants: 0 the default rule (launch_variant in render.cu); 1-5 threads
+// Render variants: 0 the default rule (below); 1-5 threads
 // per block, tree width, child order, register cap; 6 and 7 the longest-first LP
 // order (7: the ray regenerated for shading and at most 72 registers, 7 blocks
 // per SM), whose GT is variant 4's kernel.
 constexpr int kNumRenderVariants = 8;
 constexpr int kLptVariant = 6;
 constexpr int kLptVariantLean = 7;
+// Variant 0, what a session has until it is tuned: the longest-first order for
+// a session's LP casts, else the plain order in 64 registers, both with all
+// hit children of a node sorted; and in scenes of up to kPlainTris triangles the
+// plain order in 72 registers with only the nearest child put first (which
+// variant 0 was everywhere).  Measured against that everywhere: the 4K cast of the
+// 1.07 M triangle terrain 171 us for 198, its 1440p GT 345 for 385, casts of
+// terrains of 7 to 65 K triangles 97 to 142 us for 120 to 166 (since then the
+// traversal takes fewer instructions: 152 and 294 us).  In small scenes neither
+// pays: the longest-first bookkeeping costs casts of 60 to 90 us 4 to 6 us, and
+// sorting changes soups of 500 to 4,000 triangles by -15 to +13 % from scene to
+// scene.
+constexpr int kPlainTris = 4096;
 // variants that render with a longest-first order in every batch ...
 __host__ __device__ constexpr bool is_lpt_variant(int v) { return v == kLptVariant || v == kLptVariantLean; }
-// ... and those whose single-session LP casts do
-__host__ __device__ constexpr bool has_lpt_kernel(int v) { return v == 0 || is_lpt_variant(v); }
+// ... and those whose single-session LP casts of n_tris triangles do
+__host__ __device__ constexpr bool has_lpt_kernel(int v, int n_tris) {
+    return v == 0 ? n_tris > kPlainTris : is_lpt_variant(v);
+}
 // Reconstruct variants: column-run tiles (0-3), row tiles (4-7) and the
 // column-run tile with its LP footprint staged in shared memory (8).
 constexpr int kNumReconVariants = 9;
