@@ -487,7 +487,8 @@ static int vafr_build_scene_impl(const float* tri_xyz, const float* albedo_rgb, 
     if (cudaMemsetAsync(sc->status, 0, sizeof(unsigned), s) != cudaSuccess)
         return bail(fail(VAFR_ERR_CUDA, "memset status"));
     if (n > 0) {
-        // device inputs are read where they are, host inputs copied first
+        // device inputs are read where they are, host inputs and those between two
+        // floats' addresses copied first
         struct Copy {   // freed on every way out
             float* p = nullptr;
             ~Copy() { if (p) cudaFree(p); }
@@ -495,9 +496,12 @@ static int vafr_build_scene_impl(const float* tri_xyz, const float* albedo_rgb, 
         b.tris = tri_xyz;
         b.albedo = albedo_rgb;
         auto to_device = [&](Copy& c, const float** in, size_t count) -> cudaError_t {
-            if (!*in || is_device_ptr(*in)) return cudaSuccess;
+            const bool device = *in && is_device_ptr(*in);
+            if (!*in || (device && aligned(*in, sizeof(float)))) return cudaSuccess;
             cudaError_t e = cudaMalloc(&c.p, sizeof(float) * count);
-            if (e == cudaSuccess) e = cudaMemcpyAsync(c.p, *in, sizeof(float) * count, cudaMemcpyHostToDevice, s);
+            if (e == cudaSuccess)
+                e = cudaMemcpyAsync(c.p, *in, sizeof(float) * count,
+                                    device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s);
             *in = c.p;
             return e;
         };

@@ -2,6 +2,8 @@
 clustering rounds' tiles of 488, the 2,048 clusters that one block finishes,
 and more than 4,096 tiles, whose counts are scanned by a launch of their own."""
 
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -76,3 +78,28 @@ def test_binary_tree_casts_the_same_hits(V, torch_mod):
     assert torch.equal(out[0][1], out[1][1]) and torch.equal(out[0][0], out[1][0])
     V.vafr_session_destroy(s)
     V.vafr_scene_destroy(h)
+
+
+@pytest.mark.parametrize("shift", [0, 1, 2, 3, 4, 8])
+def test_device_inputs_at_any_address(V, torch_mod, shift):
+    """Triangles and albedo in device memory at any byte address build the tree of
+    host inputs."""
+    torch = torch_mod
+    sc = _soup(1000, 9, 0.05)
+    light = (ctypes.c_float * 3)(*[float(v) for v in sc.light_dir])
+    ref = V.vafr_build_scene(sc.tris.reshape(-1, 9), sc.albedo, sc.light_dir)
+    held = []
+    for x in (sc.tris, sc.albedo):
+        raw = torch.from_numpy(np.frombuffer(np.ascontiguousarray(x, np.float32).tobytes(), np.uint8).copy())
+        buf = torch.zeros(raw.numel() + 16, dtype=torch.uint8, device="cuda")
+        buf[shift:shift + raw.numel()] = raw.cuda()
+        held.append(buf)
+    torch.cuda.synchronize()
+    out = ctypes.c_void_p()
+    lib = V.load()
+    assert lib.vafr_build_scene(held[0].data_ptr() + shift, held[1].data_ptr() + shift, 1000,
+                                ctypes.cast(light, ctypes.c_void_p), None, ctypes.byref(out)) == 0
+    for a, b in zip(V.vafr_scene_export_tree4(ref), V.vafr_scene_export_tree4(out.value)):
+        assert np.array_equal(a.view(np.int32), b.view(np.int32))
+    V.vafr_scene_destroy(ref)
+    V.vafr_scene_destroy(out.value)
