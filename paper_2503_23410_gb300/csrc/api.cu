@@ -277,22 +277,29 @@ cudaError_t lpt_next(LptState* st, unsigned& frames, cudaStream_t s, LptState** 
     return cudaSuccess;
 }
 
-// Scratch of a pooled path tracing launch: the session's, allocated by the first
-// call that wants it.  NULL leaves the launch to the kernel that needs none: for
-// little work, and where the allocation fails.  The relaxed mode keeps it from
-// ending a capture that is under way, on this call's stream or another thread's.
-void* path_scratch(vafr_session* s, long long work, int depth) {
-    if (!path_uses_pool(work, depth)) return nullptr;
-    if (!s->d_path) {
-        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-        if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return nullptr;
-        if (cudaMalloc(&s->d_path, path_scratch_bytes(s->sms)) != cudaSuccess) {
-            cudaGetLastError();
-            s->d_path = nullptr;
-        }
-        cudaThreadExchangeStreamCaptureMode(&mode);
+// Scratch of a pooled path tracing launch: the session's; NULL, for the kernel that
+// needs none, for little work and until path_scratch_next has allocated it.
+void* path_scratch(const vafr_session* s, long long work, int depth) {
+    return path_uses_pool(work, depth) ? s->d_path : nullptr;
+}
+
+// After a launch that could have used the scratch: allocates it for the next one
+// while the GPU works (10 MB, some 170 us: before the first launch it made a
+// 490 us path tracing pass 530).  A failure leaves the session without.  The relaxed
+// mode keeps it from ending a capture that is under way, on this call's stream or
+// another thread's.
+void path_scratch_next(vafr_session* s, long long work, int depth) {
+    if (s->d_path || !path_uses_pool(work, depth)) return;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) {
+        cudaGetLastError();
+        return;
     }
-    return s->d_path;
+    if (cudaMalloc(&s->d_path, path_scratch_bytes(s->sms)) != cudaSuccess) {
+        cudaGetLastError();
+        s->d_path = nullptr;
+    }
+    cudaThreadExchangeStreamCaptureMode(&mode);
 }
 
 int lpt_chunks(int64_t n_texels) { return (int)((n_texels + kLptChunk - 1) / kLptChunk); }
@@ -853,6 +860,7 @@ int vafr_render_lp_pt(const vafr_scene* scene, vafr_session* s, int32_t eye_mask
     }
     void* scratch = path_scratch(s, b.total_work, max_diffuse);
     CUDA_TRY(launch_path_lp(scene->dev, b, (unsigned long long)seed, max_diffuse, scratch, as_stream(stream), s->sms));
+    path_scratch_next(s, b.total_work, max_diffuse);
     return VAFR_OK;
 }
 
@@ -1096,6 +1104,7 @@ int vafr_render_full_gt_pt(const vafr_scene* scene, vafr_session* s, int32_t eye
     b.total_work = gt_items(f);
     void* scratch = path_scratch(s, b.total_work, max_diffuse);
     CUDA_TRY(launch_path_gt(scene->dev, b, (unsigned long long)seed, max_diffuse, scratch, as_stream(stream), s->sms));
+    path_scratch_next(s, b.total_work, max_diffuse);
     return VAFR_OK;
 }
 
