@@ -573,7 +573,7 @@ def run_gpu(args, w):
                                 [os.path.join(csrc, f) for f in ("render.cu", "trace.cuh")], traffic_key)
     tr_recon, _ = _traffic("reconstruct", [os.path.join(csrc, f) for f in ("reconstruct.cu", "lp_map.cuh")],
                            traffic_key)
-    render_kernel = ("k_path_lp" if pt else
+    render_kernel = ("k_path" if pt else
                      "k_render_lp (left eye) + k_rep_* warp + k_render_list (holes)" if rep else
                      "k_render_lp_lpt" if lpt else "k_render_lp")
     roof_render = {"kernel": render_kernel, "bound": "alu",

@@ -271,15 +271,15 @@ VAFR_API int vafr_session_sizes(const vafr_session* session, int64_t* lp_bytes_p
 /* Reads (set = 0) or writes (set = 1) the kernel variants used by this
  * session's single-session calls: cfg[0] render variant, cfg[1] reconstruct
  * tile shape (see vafr_tuning_space).  Render variants 6 and 7, and the
- * default 0, take the LP work in chunks of 32 rays and render the chunks that
+ * default 0 in scenes above 4,096 triangles, take the LP work in chunks of 32 rays and render the chunks that
  * were slowest in the session's previous frame first, so a launch does not end
  * waiting for slow chunks that happened to come last (7 keeps fewer registers,
  * 7 blocks per SM).  Results do not depend on the choice.
  * Errors: INVALID_ARG (NULL, variant out of range). */
 VAFR_API int vafr_session_tuning(vafr_session* session, int32_t set, int32_t cfg[2]);
 /* Picks the session's kernel variants by timing whole frames at the current
- * gaze: every render variant renders `warm` untimed frames (variants 6 and 7,
- * the longest-first order, need two frames of history) and then `iters` timed
+ * gaze: every render variant renders `warm` untimed frames (variants 0, 6
+ * and 7, the longest-first order, need two frames of history) and then `iters` timed
  * frames (render_lp of all eyes + reconstruct of every eye, CUDA events on
  * `stream`); then every reconstruct variant is timed the same way with the
  * chosen render variant.  The fastest pair is kept and written to cfg_out
@@ -386,8 +386,8 @@ VAFR_API int vafr_rep_hole_count(vafr_session* session, int64_t* holes, void* st
  * centre ray and the depth test keeps the smallest (distance, id), so the
  * buffer equals the GT cast's closest hits (triangle parts closer than 1e-4
  * scene units to the camera plane are not drawn).  Triangles are clipped to
- * the view frustum; boxes of at most 128 pixels are rasterised one thread per
- * triangle, larger ones as 16 x 8 pixel tiles spread evenly over all warps.
+ * the view frustum; boxes of at most 96 pixels are rasterised by the warp that
+ * set their triangles up, larger ones as 16 x 8 pixel tiles handed out to all warps.
  * Scene-owned scratch (~32 B per triangle) is allocated on first use, so
  * deferred calls on one scene must not overlap.
  * vafr_render_vbuffer: the G-buffer pass of one eye into vbuf_out (device,
