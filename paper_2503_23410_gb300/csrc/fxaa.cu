@@ -228,6 +228,7 @@ __device__ __forceinline__ int find_aa_frame(const B& b, long long w) {
 // the slots past n_texels (an eye has n_texels + 2 n_cols).
 template <class B>
 __global__ void __launch_bounds__(256) k_lp_luma(const __grid_constant__ B b) {
+    after_previous();
     for (long long w = (long long)blockIdx.x * 256 + threadIdx.x; w < b.total_aa;
          w += (long long)gridDim.x * 256) {
         const FrameDesc& f = b.d[find_aa_frame(b, w)];
@@ -262,7 +263,8 @@ struct AaTexel {
 
 // Pass 2: the filter.  A block takes as many texels as it has threads, copies
 // the flat ones and lists the edges, which its first threads then filter side
-// by side.  An LP buffer in FP32 takes 38 us, both passes (47 with 256 threads,
+// by side.  An LP buffer in FP32 takes 37 us, both passes, and 33.5 since their
+// launches overlap (47 with 256 threads,
 // each filtering its own texel, a quotient at every step of the search and the
 // lumas in the work order; 40 without the list).  Larger blocks or several
 // texels to a thread lose to the densest blocks, whose searches end the launch.
@@ -273,6 +275,7 @@ __global__ void __launch_bounds__(kFilterThreads, 10) k_fxaa_lp(const __grid_con
     __shared__ unsigned short edges[kFilterThreads];
     __shared__ int n_edges;
     if (threadIdx.x == 0) n_edges = 0;
+    after_previous();
     __syncthreads();
     const long long w0 = (long long)blockIdx.x * kFilterThreads;
     const int lane = threadIdx.x & 31;
@@ -303,10 +306,10 @@ cudaError_t launch_fxaa(const B& b, cudaStream_t s, int num_sms) {
     const long long want = (b.total_aa + 255) / 256;   // one thread per texel
     const long long cap = (long long)num_sms * 64;
     const unsigned grid = (unsigned)(want < cap ? want : cap);
-    k_lp_luma<B><<<grid, 256, 0, s>>>(b);
-    k_fxaa_lp<B><<<(unsigned)((b.total_aa + kFilterThreads - 1) / kFilterThreads), kFilterThreads, 0, s>>>(b);
-    count_launch(2);
-    return cudaGetLastError();
+    const unsigned filters = (unsigned)((b.total_aa + kFilterThreads - 1) / kFilterThreads);
+    const cudaError_t e = launch_overlapped(k_lp_luma<B>, grid, 256, 0, s, b);
+    if (e != cudaSuccess) return e;
+    return launch_overlapped(k_fxaa_lp<B>, filters, kFilterThreads, 0, s, b);
 }
 
 template cudaError_t launch_fxaa<SmallBatch>(const SmallBatch&, cudaStream_t, int);

@@ -299,6 +299,7 @@ __global__ void __launch_bounds__(32 * kRasterWarps, kRasterBlocks)
 k_vbuf_raster(const SceneDev sc, const __grid_constant__ SmallBatch b, unsigned long long* vbuf, int4* big,
               int* big_leaf, long long* big_first, unsigned long long* counter, unsigned big_cap, int per,
               unsigned long long* stats) {
+    after_previous();
     __shared__ RasterWarp warps[kRasterWarps];
     __shared__ int starts[kRasterWarps][32];
     __shared__ float widths[kRasterWarps][32];   // 1 / box width
@@ -420,6 +421,7 @@ __global__ void __launch_bounds__(32 * kRasterWarps, kRasterBlocks)
 k_vbuf_tiles(const SceneDev sc, const __grid_constant__ SmallBatch b, unsigned long long* vbuf, const int4* big,
              const int* big_leaf, const long long* big_first, unsigned long long* counter, unsigned big_cap,
              unsigned long long* stats) {
+    after_previous();
     __shared__ RasterWarp warps[kRasterWarps];
     RasterWarp& w = warps[threadIdx.x >> 5];
     const FrameDesc& f = b.d[0];
@@ -554,6 +556,7 @@ __device__ __forceinline__ float4 shade_vbuf(const SceneDev& sc, const FrameDesc
 __global__ void __launch_bounds__(256)
 k_shade_lp_vbuf(const SceneDev sc, const __grid_constant__ SmallBatch b, const unsigned long long* vbuf,
                 const int* leaf_of) {
+    after_previous();
     const FrameDesc& f = b.d[0];
     for (int k = blockIdx.x * 256 + threadIdx.x; k < f.n_texels; k += gridDim.x * 256) {
         const int2 tc = __ldg(f.work + k);
@@ -576,6 +579,7 @@ k_shade_lp_vbuf(const SceneDev sc, const __grid_constant__ SmallBatch b, const u
 __global__ void __launch_bounds__(256)
 k_shade_gt_vbuf(const SceneDev sc, const __grid_constant__ SmallBatch b, const unsigned long long* vbuf,
                 const int* leaf_of) {
+    after_previous();
     const FrameDesc& f = b.d[0];
     const long long n = (long long)f.W * f.H;
     for (long long p = blockIdx.x * 256ll + threadIdx.x; p < n; p += gridDim.x * 256ll) {
@@ -607,19 +611,16 @@ cudaError_t launch_vbuffer(const SceneDev& sc, const SmallBatch& b, const VbufSc
     const int per = min(32, max(1, (sc.n_tris + blocks * kRasterWarps - 1) / (blocks * kRasterWarps)));
     const int groups = (sc.n_tris + per - 1) / per;
     const int grid = min((groups + kRasterWarps - 1) / kRasterWarps, 4 * blocks);
-    if (stats) {
-        k_vbuf_raster<true><<<grid, tpb, 0, s>>>(sc, b, v.vbuf, v.big, v.big_leaf, v.big_first, v.counter,
-                                                  v.big_cap, per, stats);
-        k_vbuf_tiles<true><<<blocks, tpb, 0, s>>>(sc, b, v.vbuf, v.big, v.big_leaf, v.big_first, v.counter,
-                                                   v.big_cap, stats);
-    } else {
-        k_vbuf_raster<false><<<grid, tpb, 0, s>>>(sc, b, v.vbuf, v.big, v.big_leaf, v.big_first, v.counter,
-                                                   v.big_cap, per, nullptr);
-        k_vbuf_tiles<false><<<blocks, tpb, 0, s>>>(sc, b, v.vbuf, v.big, v.big_leaf, v.big_first, v.counter,
-                                                    v.big_cap, nullptr);
-    }
-    count_launch(2);
-    return cudaGetLastError();
+    if (stats)
+        k_vbuf_raster<true><<<grid, tpb, 0, s>>>(sc, b, v.vbuf, v.big, v.big_leaf, v.big_first, v.counter, v.big_cap,
+                                                  per, stats);
+    else
+        k_vbuf_raster<false><<<grid, tpb, 0, s>>>(sc, b, v.vbuf, v.big, v.big_leaf, v.big_first, v.counter, v.big_cap,
+                                                   per, nullptr);
+    count_launch(1);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    return launch_overlapped(stats ? k_vbuf_tiles<true> : k_vbuf_tiles<false>, (unsigned)blocks, tpb, 0, s, sc, b, v.vbuf,
+                             v.big, v.big_leaf, v.big_first, v.counter, v.big_cap, stats);
 }
 
 cudaError_t launch_leaf_of(const SceneDev& sc, int* leaf_of, cudaStream_t s, int num_sms) {
@@ -633,12 +634,11 @@ cudaError_t launch_shade_vbuf(const SceneDev& sc, const SmallBatch& b, const uns
                               const int* leaf_of, bool full_res, cudaStream_t s, int num_sms) {
     if (full_res) {
         const long long n = (long long)b.d[0].W * b.d[0].H;
-        k_shade_gt_vbuf<<<(unsigned)min((n + 255) / 256, (long long)num_sms * 16), 256, 0, s>>>(sc, b, vbuf, leaf_of);
-    } else {
-        k_shade_lp_vbuf<<<(unsigned)min((b.d[0].n_texels + 255) / 256, num_sms * 16), 256, 0, s>>>(sc, b, vbuf, leaf_of);
+        return launch_overlapped(k_shade_gt_vbuf, (unsigned)min((n + 255) / 256, (long long)num_sms * 16), 256, 0, s, sc, b,
+                                 vbuf, leaf_of);
     }
-    count_launch(1);
-    return cudaGetLastError();
+    return launch_overlapped(k_shade_lp_vbuf, (unsigned)min((b.d[0].n_texels + 255) / 256, num_sms * 16), 256, 0, s, sc, b,
+                             vbuf, leaf_of);
 }
 
 }  // namespace vafr

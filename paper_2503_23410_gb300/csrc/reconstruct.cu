@@ -170,6 +170,7 @@ k_reconstruct(const __grid_constant__ B b) {
     const int tile = (int)blockIdx.x;
     if (threadIdx.x == 0) stage_frame(b, tile, sh);
     __syncthreads();
+    after_previous();
     const ReconRegs f = sh.r;
     const int W = sh.W, H = sh.H;
     void* const disp = sh.disp;
@@ -531,6 +532,7 @@ k_reconstruct_runs(const __grid_constant__ B b) {
     const int tile = (int)blockIdx.x;
     if (threadIdx.x == 0) stage_frame(b, tile, sh);
     __syncthreads();
+    after_previous();
     const ReconRegs f = sh.r;
     const int W = sh.W, H = sh.H;
     const int local = tile - sh.tile_begin;
@@ -561,9 +563,7 @@ k_reconstruct_runs(const __grid_constant__ B b) {
 template <int TW, int R, int LW, int MINB, bool REUSE_U, class B>
 cudaError_t launch_runs(const B& b, cudaStream_t s) {
     if (b.total_tiles <= 0) return cudaSuccess;
-    k_reconstruct_runs<TW, R, LW, MINB, REUSE_U, B><<<(unsigned)b.total_tiles, TW, 0, s>>>(b);
-    count_launch(1);
-    return cudaGetLastError();
+    return launch_overlapped(k_reconstruct_runs<TW, R, LW, MINB, REUSE_U, B>, (unsigned)b.total_tiles, TW, 0, s, b);
 }
 
 // Column-run tile (TW threads, one display column each, R rows) whose LP
@@ -578,6 +578,7 @@ k_reconstruct_staged(const __grid_constant__ B b) {
     const int tile = (int)blockIdx.x;
     if (threadIdx.x == 0) stage_frame(b, tile, sh);
     __syncthreads();
+    after_previous();
     const ReconRegs f = sh.r;
     const int W = sh.W, H = sh.H;
     const int local = tile - sh.tile_begin;
@@ -616,17 +617,13 @@ k_reconstruct_staged(const __grid_constant__ B b) {
 template <int TW, int R, int MINB, class B>
 cudaError_t launch_staged(const B& b, cudaStream_t s) {
     if (b.total_tiles <= 0) return cudaSuccess;
-    k_reconstruct_staged<TW, R, MINB, B><<<(unsigned)b.total_tiles, TW, 0, s>>>(b);
-    count_launch(1);
-    return cudaGetLastError();
+    return launch_overlapped(k_reconstruct_staged<TW, R, MINB, B>, (unsigned)b.total_tiles, TW, 0, s, b);
 }
 
 template <int TW, int TH, int PX, class B>
 cudaError_t launch_shape(const B& b, cudaStream_t s) {
     if (b.total_tiles <= 0) return cudaSuccess;
-    k_reconstruct<TW, TH, PX, B><<<(unsigned)b.total_tiles, (TW / PX) * TH, 0, s>>>(b);
-    count_launch(1);
-    return cudaGetLastError();
+    return launch_overlapped(k_reconstruct<TW, TH, PX, B>, (unsigned)b.total_tiles, (TW / PX) * TH, 0, s, b);
 }
 
 }  // namespace

@@ -52,6 +52,7 @@ k_render_lp(const SceneDev sc, const __grid_constant__ B b) {
 // the 8K binocular VaFR_Rep cast 488 -> 453 us (8 rays 463, 16 rays 474).
 __global__ void __launch_bounds__(128)
 k_render_list(const SceneDev sc, const __grid_constant__ SmallBatch b, const unsigned* count) {
+    after_previous();
     const int lane = threadIdx.x & 31;
     const long long total = (long long)*count;
     const FrameDesc& f = b.d[0];
@@ -358,9 +359,7 @@ cudaError_t launch_render_list(const SceneDev& scene, const SmallBatch& batch, c
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_render_list, 128, 0);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
-    k_render_list<<<(unsigned)(per_sm * num_sms), 128, 0, s>>>(scene, batch, count);
-    count_launch(1);
-    return cudaGetLastError();
+    return launch_overlapped(k_render_list, (unsigned)(per_sm * num_sms), 128, 0, s, scene, batch, count);
 }
 
 cudaError_t launch_render_stats(const SceneDev& scene, const SmallBatch& batch,

@@ -88,6 +88,7 @@ __global__ void __launch_bounds__(256) k_rep_vertices(const __grid_constant__ Sm
     const FrameDesc& L = b.d[0];
     const FrameDesc& R = b.d[1];
     float4* const vert = r.vert;
+    after_previous();
     const int slots = R.n_texels + guards(R.n_cols) - 1;
     for (int k = blockIdx.x * 256 + threadIdx.x; k < slots; k += gridDim.x * 256) r.zbuf[k] = kEmptyKey;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -200,6 +201,7 @@ __device__ __forceinline__ bool load_tri(const float4* vert, const int tv[3], fl
 // occupancy; with 48 registers they spill, 6 us slower).
 __global__ void __launch_bounds__(256)
 k_rep_raster(const __grid_constant__ SmallBatch b, const float4* vert, unsigned long long* zbuf) {
+    after_previous();
     const FrameDesc& L = b.d[0];
     const FrameDesc& R = b.d[1];
     const int C = R.n_cols;
@@ -270,6 +272,7 @@ k_rep_resolve(const __grid_constant__ SmallBatch b, const float4* vert, const un
     const FrameDesc& L = b.d[0];
     const FrameDesc& R = b.d[1];
     const int C = L.n_cols;
+    after_previous();
     __shared__ unsigned warp_off[8];
     __shared__ unsigned block_base;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -351,11 +354,11 @@ cudaError_t launch_reproject(const SmallBatch& b, const RepScratch& r, cudaStrea
     const unsigned grid = (unsigned)min((b.d[0].n_texels + 255) / 256, num_sms * 16);
     const unsigned rgrid =
         (unsigned)max(1, min((R.n_texels + 256 * kResolveItems - 1) / (256 * kResolveItems), num_sms * 64));
-    k_rep_vertices<<<grid, 256, 0, s>>>(b, r);
-    k_rep_raster<<<grid, 256, 0, s>>>(b, r.vert, r.zbuf);
-    k_rep_resolve<<<rgrid, 256, 0, s>>>(b, r.vert, r.zbuf, r.holes, r.count, r.tri_out);
-    count_launch(3);
-    return cudaGetLastError();
+    cudaError_t e = launch_overlapped(k_rep_vertices, grid, 256, 0, s, b, r);
+    if (e == cudaSuccess) e = launch_overlapped(k_rep_raster, grid, 256, 0, s, b, r.vert, r.zbuf);
+    if (e == cudaSuccess)
+        e = launch_overlapped(k_rep_resolve, rgrid, 256, 0, s, b, r.vert, r.zbuf, r.holes, r.count, r.tri_out);
+    return e;
 }
 
 }  // namespace vafr

@@ -138,30 +138,6 @@ __device__ __forceinline__ void make_node(const Ploc& p, int id, float4 a, float
     lo.w = __int_as_float(id);
 }
 
-// The rounds' launches overlap their start-up: a kernel is put on the SMs while
-// the one before it is finishing, and waits for its results here.
-__device__ __forceinline__ void after_previous() {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-
-template <class... P, class... A>
-cudaError_t launch_overlapped(void (*kernel)(P...), unsigned grid, unsigned block, size_t shared, cudaStream_t s,
-                              A... args) {
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(block);
-    cfg.dynamicSmemBytes = shared;
-    cfg.stream = s;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    count_launch(1);
-    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
-}
-
 // First launch of a round: each cluster's fate and each tile's counts.  A
 // thread takes one position from 2 kRadius before the tile on (the clusters'
 // neighbours' neighbours decide with it).  Blocks stride over the tiles, so
