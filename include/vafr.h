@@ -388,7 +388,7 @@ VAFR_API int vafr_rep_hole_count(vafr_session* session, int64_t* holes, void* st
  * scene units to the camera plane are not drawn).  Triangles are clipped to
  * the view frustum; boxes of at most 96 pixels are rasterised by the warp that
  * set their triangles up, larger ones as 16 x 8 pixel tiles handed out to all warps.
- * Scene-owned scratch (~32 B per triangle) is allocated on first use, so
+ * The scene owns the scratch (32 B per triangle, where its build's was), so
  * deferred calls on one scene must not overlap.
  * vafr_render_vbuffer: the G-buffer pass of one eye into vbuf_out (device,
  *   height x width uint64, 8-byte aligned).

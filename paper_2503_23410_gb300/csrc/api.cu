@@ -123,7 +123,10 @@ struct vafr_scene {
     bool injected = false;         // vafr_scene_inject_fault: root references and keys saved
     int4 root_refs{}, root_keys{};
     float4* d_plights = nullptr;   // point lights (vafr_scene_set_point_lights)
-    // deferred path scratch (first use): triangle id -> leaf, large-triangle list
+    // deferred path scratch, where the build's was (as much as four arrays of it, so that
+    // a scene's first visibility buffer waits for no allocation): triangle id -> leaf,
+    // filled by the first use, and the large-triangle list
+    bool leaf_of_ready = false;
     int* d_leaf_of = nullptr;
     int4* d_big = nullptr;
     int* d_big_leaf = nullptr;
@@ -456,6 +459,7 @@ static int vafr_build_scene_impl(const float* tri_xyz, const float* albedo_rgb, 
     auto carve = [&] {
         at = 0;
         take(&sc->status, 1);
+        take(&sc->d_n_big, 2);
         if (n == 0) return;
         take(&b.codes, N);
         take(&b.ids, N);
@@ -467,10 +471,12 @@ static int vafr_build_scene_impl(const float* tri_xyz, const float* albedo_rgb, 
         take(&b.child, NI);          // lbvh_hierarchy
         take(&b.node_box, 6 * NI);
         take(&b.nodes, 4 * NI);
-        take(&b.links, NI);
+        take(&b.links, N);           // from here and keys_sorted: also the deferred path's scratch
         take(&b.leaf_parent, N);
-        take(&b.flags, N);
-        take(&b.climbers, N);
+        long long* pairs = nullptr;
+        take(&pairs, N);
+        b.flags = reinterpret_cast<unsigned*>(pairs);
+        b.climbers = pairs ? reinterpret_cast<int32_t*>(pairs) + N : nullptr;
         size_t end = at;
         at = from;                   // lbvh_sort, tree4_build and tree4_pack
         take(&b.clusters, 2 * N);
@@ -536,6 +542,10 @@ static int vafr_build_scene_impl(const float* tri_xyz, const float* albedo_rgb, 
     d.nodes4 = b.nodes4;
     d.n_nodes4 = sc->n_nodes4;
     d.leaves = b.leaves;
+    sc->d_leaf_of = reinterpret_cast<int*>(b.keys_sorted);
+    sc->d_big = b.links;
+    sc->d_big_leaf = b.leaf_parent;
+    sc->d_big_first = reinterpret_cast<long long*>(b.flags);
     d.albedo = b.albedo4;
     d.n_tris = n;
     d.root = n == 0 ? INT_MIN : (n == 1 ? ~0 : 0);
@@ -959,15 +969,11 @@ int vafr_rep_hole_count(vafr_session* s, int64_t* holes, void* stream) {
 // ---- deferred path -----------------------------------------------------------------
 static int deferred_scratch(const vafr_scene* scene_c, cudaStream_t st) {
     auto* scene = const_cast<vafr_scene*>(scene_c);
-    if (scene->d_leaf_of) return VAFR_OK;
-    const size_t n = (size_t)(scene->n > 0 ? scene->n : 1);
-    int rc = scene->alloc(&scene->d_leaf_of, n);
-    if (!rc) rc = scene->alloc(&scene->d_big, n);
-    if (!rc) rc = scene->alloc(&scene->d_big_leaf, n);
-    if (!rc) rc = scene->alloc(&scene->d_big_first, n);
-    if (!rc) rc = scene->alloc(&scene->d_n_big, 2);
-    if (rc) return fail(VAFR_ERR_OOM, "deferred scratch");
+    if (scene->leaf_of_ready) return VAFR_OK;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    CUDA_TRY(cudaStreamIsCapturing(st, &capture));
     CUDA_TRY(launch_leaf_of(scene->dev, scene->d_leaf_of, st, scene->sms));
+    scene->leaf_of_ready = capture == cudaStreamCaptureStatusNone;   // a captured launch has filled nothing yet
     return VAFR_OK;
 }
 

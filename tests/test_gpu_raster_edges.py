@@ -37,3 +37,45 @@ def test_equals_the_cast(V, torch_mod, width, height, n, size):
     assert stats["prefilter"] >= stats["filtered"] >= stats["tests"] >= stats["atomics"] >= int((ids >= 0).sum())
     V.vafr_session_destroy(s)
     V.vafr_scene_destroy(h)
+
+
+def test_first_call_inside_a_capture(V, torch_mod):
+    """A scene's first visibility buffer and shading may be captured; eager calls
+    before and after the replay give the bits of an uncaptured scene."""
+    torch = torch_mod
+    sc = random_triangles_scene(500, seed=3)
+    pose = np.array([[1, 0, 0, 0], [0, 1, 0, 0], [0, 0, 1, -3.0]])
+    out = []
+    for captured in (False, True):
+        h, keep = device_scene(V, sc, torch)
+        s = V.vafr_session_create(V.make_session_desc(200, 150, 70.0, [pose]))
+        V.vafr_set_gaze(s, 0, 90.0, 70.0)
+        slots = V.vafr_session_sizes(s)[0] // 16
+        vbuf = torch.zeros(200 * 150, dtype=torch.int64, device="cuda")
+        lp = torch.zeros((slots, 4), dtype=torch.float32, device="cuda")
+        torch.cuda.synchronize()
+
+        def frame(stream=None):
+            V.vafr_render_vbuffer(h, s, 0, vbuf, stream)
+            V.vafr_shade_lp_deferred(h, s, 0, vbuf, lp, stream)
+
+        if captured:
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g):
+                frame(torch.cuda.current_stream().cuda_stream)
+            frame()
+            torch.cuda.synchronize()
+            out.append((vbuf.clone(), lp.clone()))
+            vbuf.zero_()
+            lp.zero_()
+            g.replay()
+        else:
+            frame()
+        torch.cuda.synchronize()
+        assert V.vafr_session_check(s) == 0
+        out.append((vbuf.clone(), lp.clone()))
+        V.vafr_session_destroy(s)
+        V.vafr_scene_destroy(h)
+    assert (out[0][0] != -1).any()
+    for vb, lp in out[1:]:
+        assert torch.equal(vb, out[0][0]) and torch.equal(lp, out[0][1])
