@@ -752,6 +752,7 @@ static int vafr_session_create_impl(const vafr_session_desc* desc, vafr_session*
     if (d.lp_fxaa && (e = cudaMalloc(&s->d_luma, sizeof(float) * s->n_slots * d.n_eyes)) != cudaSuccess)
         return bail(e);
     for (int eye = 0; eye < d.n_eyes; ++eye) fill_static(s.get(), eye);
+    prepare_render();
     *out = s.release();
     return VAFR_OK;
 }

@@ -296,11 +296,6 @@ cudaError_t launch_one(const SceneDev& sc, const B& b, cudaStream_t s, int num_s
 template <int TPB, int ORDER, bool REGEN = false, int MINB = 1, class B>
 cudaError_t launch_lpt(const SceneDev& sc, const B& b, cudaStream_t s, int num_sms) {
     auto kern = k_render_lp_lpt<TPB, ORDER, B, REGEN, MINB>;
-    // the kernel's few bytes of shared memory must not shrink the L1 the
-    // traversal lives in: ask for the smallest shared-memory carveout
-    static const cudaError_t carve =
-        cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
-    if (carve != cudaSuccess) return carve;
     int per_sm = 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, TPB, 0);
     if (e != cudaSuccess) return e;
@@ -335,7 +330,21 @@ cudaError_t launch_variant(const SceneDev& sc, const B& b, int variant, cudaStre
         default: return launch_lpt<128, 0, true, 7>(sc, b, s, sms);
     }
 }
+
+// The longest-first kernels' few bytes of shared memory must not shrink the L1 the
+// traversal lives in: they ask for the smallest shared-memory carveout.
+template <class B>
+void ask_for_l1() {
+    cudaFuncSetAttribute(k_render_lp_lpt<128, 0, B, false, 1>, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
+    cudaFuncSetAttribute(k_render_lp_lpt<128, 0, B, true, 7>, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
+}
 }  // namespace
+
+void prepare_render() {
+    ask_for_l1<SmallBatch>();
+    ask_for_l1<BigBatch>();
+    cudaGetLastError();   // hints: without them the casts only take longer
+}
 
 template <class B>
 cudaError_t launch_render_lp(const SceneDev& scene, const B& batch, int variant, cudaStream_t s,

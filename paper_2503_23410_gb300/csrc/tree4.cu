@@ -696,8 +696,9 @@ cudaError_t tree4_build(const LbvhBuffers& b, void* scratch, cudaStream_t s, int
     p.fates = sc.fates;
     p.counts = sc.counts;
     p.state = sc.state;
-    static const cudaError_t big = cudaFuncSetAttribute(k_ploc_tail, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                        (int)sizeof(TailShared));
+    // the attribute is the current device's and context's: every build sets it
+    const cudaError_t big = cudaFuncSetAttribute(k_ploc_tail, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 (int)sizeof(TailShared));
     if (big != cudaSuccess) return big;
     k_ploc_start<<<1, 1, 0, s>>>(sc.state, n);
     count_launch(1);

@@ -169,6 +169,9 @@ constexpr int kNumReconVariants = 9;
 struct ReconShape { int tw, th; int px; };
 ReconShape recon_shape(int variant);
 
+// Sets the render kernels' attributes for the current device and context; every
+// session does (they are kept neither across devices nor across a device reset).
+void prepare_render();
 template <class B>
 cudaError_t launch_render_lp(const SceneDev& scene, const B& batch, int variant,
                              cudaStream_t s, int num_sms);
