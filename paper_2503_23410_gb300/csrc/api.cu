@@ -1072,7 +1072,7 @@ int vafr_fxaa_lp(vafr_session* s, int32_t eye, const void* lp, void* lp_out, voi
     b.d[0] = f;
     b.n = 1;
     b.total_aa = s->n_texels;
-    CUDA_TRY(launch_fxaa(b, as_stream(stream), s->sms));
+    CUDA_TRY(launch_fxaa(b, as_stream(stream)));
     return VAFR_OK;
 }
 
@@ -1165,7 +1165,7 @@ int vafr_render_frame(const vafr_scene* scene, vafr_session* s, void* display_ou
         b.total_tiles += recon_tiles(f, s->recon_variant);
         b.d[b.n++] = f;
     }
-    CUDA_TRY(launch_fxaa(b, as_stream(stream), s->sms));
+    CUDA_TRY(launch_fxaa(b, as_stream(stream)));
     CUDA_TRY(launch_reconstruct(b, s->recon_variant, as_stream(stream)));
     if (copy_out)
         CUDA_TRY(cudaMemcpyAsync(display_out, target, (size_t)dpb * eyes, cudaMemcpyDeviceToHost,
@@ -1304,7 +1304,7 @@ static int build_batch(vafr_batch* bt, const vafr_frame_desc* frames, int32_t n,
 
 static int launch_batch(vafr_batch* bt, const BigBatch& b, cudaStream_t st) {
     CUDA_TRY(launch_render_lp(bt->scene->dev, b, bt->render_variant, st, bt->scene->sms));
-    CUDA_TRY(launch_fxaa(b, st, bt->scene->sms));
+    CUDA_TRY(launch_fxaa(b, st));
     CUDA_TRY(launch_reconstruct(b, bt->recon_variant, st));
     for (const auto& c : bt->copies)
         CUDA_TRY(cudaMemcpyAsync(c.dst, c.src, c.bytes, cudaMemcpyDeviceToHost, st));

@@ -223,19 +223,38 @@ __device__ __forceinline__ int find_aa_frame(const B& b, long long w) {
     return lo;
 }
 
-// Pass 1: the luma of every slot into the frame's scratch, in slot order: the
-// thread of the i-th texel takes slot i, and those of the first 2 n_cols also
-// the slots past n_texels (an eye has n_texels + 2 n_cols).
+// Pass 1: the luma of every slot into the frame's scratch.  A block takes rows of
+// one column (blockIdx.x; frame blockIdx.z), kLumaItems to a thread and all of them
+// loaded before the first is stored; the guard slots get the lumas of the texels
+// that they stand for, whatever the buffer's own guards hold.  It reads 17 MB and
+// writes 4 for an eye in FP32, so what counts is loads in flight: both passes take
+// 31.8 us with 128 threads of 8 rows, 32.1 with 256 of 4, 32.7 with 128 of 4, 35.5 with
+// 256 of one, all on one buffer; 33.5 over buffers in turn, where a pass over the
+// slots in order, which cannot tell a guard from a texel, took 33.2.
+constexpr int kLumaThreads = 128, kLumaItems = 8, kLumaParts = 2;
+
 template <class B>
-__global__ void __launch_bounds__(256) k_lp_luma(const __grid_constant__ B b) {
+__global__ void __launch_bounds__(kLumaThreads) k_lp_luma(const __grid_constant__ B b) {
+    const FrameDesc& f = b.d[blockIdx.z];
+    if (!f.lp_aa || (int)blockIdx.x >= f.n_cols) return;
+    const int2 cc = __ldg(f.col + blockIdx.x);   // the layout's, which no launch writes
+    const int n = cc.y;
     after_previous();
-    for (long long w = (long long)blockIdx.x * 256 + threadIdx.x; w < b.total_aa;
-         w += (long long)gridDim.x * 256) {
-        const FrameDesc& f = b.d[find_aa_frame(b, w)];
-        const int i = (int)(w - f.aa_begin);
-        f.luma[i] = luma_of(ld_texel(f.lp, f.lp_fmt, i));
-        for (int k = i; k < 2 * f.n_cols; k += f.n_texels)
-            f.luma[f.n_texels + k] = luma_of(ld_texel(f.lp, f.lp_fmt, f.n_texels + k));
+    for (int j0 = (int)blockIdx.y * (kLumaThreads * kLumaItems) + (int)threadIdx.x; j0 < n;
+         j0 += kLumaParts * kLumaThreads * kLumaItems) {
+        float4 v[kLumaItems];
+#pragma unroll
+        for (int k = 0; k < kLumaItems; ++k)
+            if (j0 + k * kLumaThreads < n) v[k] = ld_texel(f.lp, f.lp_fmt, cc.x + j0 + k * kLumaThreads);
+#pragma unroll
+        for (int k = 0; k < kLumaItems; ++k) {
+            const int j = j0 + k * kLumaThreads;
+            if (j >= n) break;
+            const float y = luma_of(v[k]);
+            f.luma[cc.x + j] = y;
+            if (j == 0) f.luma[cc.x + n] = y;
+            if (j == n - 1) f.luma[cc.x - 1] = y;
+        }
     }
 }
 
@@ -301,18 +320,17 @@ __global__ void __launch_bounds__(kFilterThreads, 10) k_fxaa_lp(const __grid_con
 }  // namespace
 
 template <class B>
-cudaError_t launch_fxaa(const B& b, cudaStream_t s, int num_sms) {
+cudaError_t launch_fxaa(const B& b, cudaStream_t s) {
     if (b.total_aa <= 0) return cudaSuccess;
-    const long long want = (b.total_aa + 255) / 256;   // one thread per texel
-    const long long cap = (long long)num_sms * 64;
-    const unsigned grid = (unsigned)(want < cap ? want : cap);
+    int cols = 0;
+    for (int k = 0; k < b.n; ++k) cols = max(cols, b.d[k].n_cols);
     const unsigned filters = (unsigned)((b.total_aa + kFilterThreads - 1) / kFilterThreads);
-    const cudaError_t e = launch_overlapped(k_lp_luma<B>, grid, 256, 0, s, b);
+    const cudaError_t e = launch_overlapped(k_lp_luma<B>, dim3(cols, kLumaParts, b.n), kLumaThreads, 0, s, b);
     if (e != cudaSuccess) return e;
     return launch_overlapped(k_fxaa_lp<B>, filters, kFilterThreads, 0, s, b);
 }
 
-template cudaError_t launch_fxaa<SmallBatch>(const SmallBatch&, cudaStream_t, int);
-template cudaError_t launch_fxaa<BigBatch>(const BigBatch&, cudaStream_t, int);
+template cudaError_t launch_fxaa<SmallBatch>(const SmallBatch&, cudaStream_t);
+template cudaError_t launch_fxaa<BigBatch>(const BigBatch&, cudaStream_t);
 
 }  // namespace vafr

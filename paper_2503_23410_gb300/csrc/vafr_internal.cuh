@@ -228,7 +228,7 @@ cudaError_t launch_shade_vbuf(const SceneDev& sc, const SmallBatch& b, const uns
                               const int* leaf_of, bool full_res, cudaStream_t s, int num_sms);
 // FXAA inside the LP buffer of every frame with lp_aa set (fxaa.cu).
 template <class B>
-cudaError_t launch_fxaa(const B& batch, cudaStream_t s, int num_sms);
+cudaError_t launch_fxaa(const B& batch, cudaStream_t s);
 cudaError_t launch_render_stats(const SceneDev& scene, const SmallBatch& batch,
                                 unsigned long long* counters, cudaStream_t s, int num_sms);
 
@@ -247,13 +247,13 @@ __device__ __forceinline__ void after_previous() {
 }
 
 template <class... P, class... A>
-cudaError_t launch_overlapped(void (*kernel)(P...), unsigned grid, unsigned block, size_t shared, cudaStream_t s,
+cudaError_t launch_overlapped(void (*kernel)(P...), dim3 grid, unsigned block, size_t shared, cudaStream_t s,
                               const A&... args) {
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(grid);
+    cfg.gridDim = grid;
     cfg.blockDim = dim3(block);
     cfg.dynamicSmemBytes = shared;
     cfg.stream = s;
