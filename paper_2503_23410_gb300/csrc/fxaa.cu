@@ -38,12 +38,12 @@ constexpr int kFxaaSteps = 12;
 
 __device__ __forceinline__ float4 ld_texel(const void* lp, int fmt, int slot) {
     if (fmt == VAFR_FMT_RGBA16F) {
-        const uint2 p = __ldg(reinterpret_cast<const uint2*>(lp) + slot);
+        const uint2 p = reinterpret_cast<const uint2*>(lp)[slot];
         const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&p.x));
         const float2 b = __half22float2(*reinterpret_cast<const __half2*>(&p.y));
         return make_float4(a.x, a.y, b.x, b.y);
     }
-    return __ldg(reinterpret_cast<const float4*>(lp) + slot);
+    return reinterpret_cast<const float4*>(lp)[slot];
 }
 
 __device__ __forceinline__ void st_texel(void* lp, int fmt, int slot, float4 v) {
@@ -100,7 +100,7 @@ struct Grid {
                                : (num < (1ull << 32) ? div((unsigned)num) : (int)(num / div.D));
         return cc.x + j2 + dj;
     }
-    __device__ __forceinline__ float luma(int slot) const { return __ldg(lum + slot); }
+    __device__ __forceinline__ float luma(int slot) const { return lum[slot]; }
 };
 
 __device__ __forceinline__ float abs_second_diff(float a, float b, float m) {

@@ -447,17 +447,17 @@ k_vbuf_tiles(const SceneDev sc, const __grid_constant__ SmallBatch b, unsigned l
         while (hi - lo > 1) {
             const long long step = (hi - lo + 31) / 32;
             const long long at = lo + step * (lane + 1);
-            const int below = __popc(__ballot_sync(full, at < hi && __ldg(big_first + at) <= g));
+            const int below = __popc(__ballot_sync(full, at < hi && big_first[at] <= g));
             lo += step * below;
             hi = min(hi, lo + step);
         }
         // the triangles of these tiles, one to a lane
         const long long rec = lo + lane;
-        const long long first = rec < n_rec ? __ldg(big_first + rec) : LLONG_MAX;
+        const long long first = rec < n_rec ? big_first[rec] : LLONG_MAX;
         int ntx = 0, nt = 0;   // tiles per row of the box, tiles; 0: not to be drawn
         if (first < end) {
-            const int4 bx = __ldg(big + rec);
-            const int k = __ldg(big_leaf + rec);
+            const int4 bx = big[rec];
+            const int k = big_leaf[rec];
             if (k >= 0 && k < sc.n_tris && bx.x >= 0 && bx.y >= 0 && bx.x <= bx.z && bx.y <= bx.w && bx.z < f.W &&
                 bx.w < f.H) {
                 const float4 a = __ldg(sc.leaves + 3ll * k), bb = __ldg(sc.leaves + 3ll * k + 1),
@@ -546,7 +546,7 @@ __device__ __forceinline__ float4 shade_vbuf(const SceneDev& sc, const FrameDesc
     } else {
         h.id = (int)(unsigned)(key & 0xffffffffu);
         h.t = __uint_as_float((unsigned)(key >> 32));
-        h.leaf = __ldg(leaf_of + h.id);
+        h.leaf = leaf_of[h.id];
     }
     return shade(sc, r, h);
 }

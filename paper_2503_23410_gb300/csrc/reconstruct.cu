@@ -38,11 +38,11 @@ struct px2 {
 __device__ __forceinline__ px2 load_lp(const void* lp, int fmt, int idx) {
     px2 r;
     if (fmt == VAFR_FMT_RGBA16F) {
-        const uint2 p = __ldg(reinterpret_cast<const uint2*>(lp) + idx);
+        const uint2 p = reinterpret_cast<const uint2*>(lp)[idx];
         r.rg = __half22float2(*reinterpret_cast<const __half2*>(&p.x));
         r.ba = __half22float2(*reinterpret_cast<const __half2*>(&p.y));
     } else {
-        const float4 q = __ldg(reinterpret_cast<const float4*>(lp) + idx);
+        const float4 q = reinterpret_cast<const float4*>(lp)[idx];
         r.rg = make_float2(q.x, q.y);
         r.ba = make_float2(q.z, q.w);
     }
@@ -338,9 +338,9 @@ __device__ __forceinline__ void stage_copy(const ReconRegs& f, const StagePlan& 
         const int n = ci.y - ci.x + 1, to = ci.x + ci.z;
         for (int q = lane; q < n; q += 32) {
             if (h16)
-                reinterpret_cast<uint2*>(buf)[to + q] = __ldg(reinterpret_cast<const uint2*>(f.lp) + ci.x + q);
+                reinterpret_cast<uint2*>(buf)[to + q] = reinterpret_cast<const uint2*>(f.lp)[ci.x + q];
             else
-                reinterpret_cast<float4*>(buf)[to + q] = __ldg(reinterpret_cast<const float4*>(f.lp) + ci.x + q);
+                reinterpret_cast<float4*>(buf)[to + q] = reinterpret_cast<const float4*>(f.lp)[ci.x + q];
         }
     }
 }
@@ -403,9 +403,9 @@ __device__ __forceinline__ void store_px(void* disp, long long idx, px2 v) {
         __stcs(reinterpret_cast<float4*>(disp) + idx, make_float4(v.rg.x, v.rg.y, v.ba.x, v.ba.y));
 }
 
-// Predicated loads: when `p` is false nothing is read and `v` keeps its value,
-// without a branch (the index bookkeeping of a run is branch-free); FP16 LP
-// texels, which need widening after the load, take a branch instead.
+// Predicated loads of the layout's tables: when `p` is false nothing is read and
+// `v` keeps its value, without a branch (the index bookkeeping of a run is
+// branch-free).
 __device__ __forceinline__ void ld_if(bool p, const float4* ptr, float4& v) {
     asm("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %4, 0;\n\t"
         "@q ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%5];\n\t}"
@@ -420,18 +420,13 @@ __device__ __forceinline__ void ld_if(bool p, const int4* ptr, int4& v) {
         : "r"((int)p), "l"(ptr));
 }
 
-// LP texel `idx` into `v` if `p`: FP32 RGBA, or FP16 RGBA widened exactly.
+// LP texel `idx` into `v` if `p`: FP32 RGBA, or FP16 RGBA widened exactly.  A plain
+// load, as the launch before may have written the texels (predicated inline
+// assembly, ordinary or volatile, takes the same 33.0 us for a 4K FP32 eye; through
+// the read-only path it took 32.7).
 template <int LPF>
 __device__ __forceinline__ void ld_texel_if(bool p, const void* lp, int idx, px2& v) {
-    if (LPF == VAFR_FMT_RGBA16F) {
-        // a branch: predicated-off widening instructions would still issue
-        if (p) v = load_lp(lp, LPF, idx);
-    } else {
-        asm("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %4, 0;\n\t"
-            "@q ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%5];\n\t}"
-            : "+f"(v.rg.x), "+f"(v.rg.y), "+f"(v.ba.x), "+f"(v.ba.y)
-            : "r"((int)p), "l"(reinterpret_cast<const float4*>(lp) + idx));
-    }
+    if (p) v = load_lp(lp, LPF, idx);
 }
 
 // R rows (FULL) or the first `nrows` of them, of display column x.  The

@@ -67,7 +67,7 @@ k_render_list(const SceneDev sc, const __grid_constant__ SmallBatch b, const uns
         if (lane < take && w < total) {
             Ray r;
             int glo, ghi;
-            const int t = lp_ray(f, (int)w, r, glo, ghi);
+            const int t = lp_ray(f, f.work[w], r, glo, ghi);   // listed by the launch before
             ray_setup(r);
             Hit h;
             const unsigned fault = traverse<4, false>(sc, r, h, nullptr, nullptr, nullptr);

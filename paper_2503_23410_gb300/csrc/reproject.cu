@@ -40,12 +40,12 @@ constexpr float kMaxFSpan = 0.25f;
 
 __device__ __forceinline__ float4 ld_rgba(const void* lp, int fmt, int slot) {
     if (fmt == VAFR_FMT_RGBA16F) {
-        const uint2 p = __ldg(reinterpret_cast<const uint2*>(lp) + slot);
+        const uint2 p = reinterpret_cast<const uint2*>(lp)[slot];
         const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&p.x));
         const float2 b = __half22float2(*reinterpret_cast<const __half2*>(&p.y));
         return make_float4(a.x, a.y, b.x, b.y);
     }
-    return __ldg(reinterpret_cast<const float4*>(lp) + slot);
+    return reinterpret_cast<const float4*>(lp)[slot];
 }
 
 __device__ __forceinline__ void st_rgba(void* lp, int fmt, int slot, float4 v) {
@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(256) k_rep_vertices(const __grid_constant__ Sm
         int slot, col;
         float3 o, d;
         lp_dir(L, k, slot, col, o, d);
-        const float t = __ldg(L.depth + slot);
+        const float t = L.depth[slot];
         const bool inf = !(t < INFINITY);
         float3 P;
         if (inf) {

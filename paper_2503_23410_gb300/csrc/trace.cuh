@@ -541,15 +541,13 @@ __device__ __forceinline__ int find_frame(const B& b, long long w, bool tiles) {
     return lo;
 }
 
-// LP ray of the frame's work item k (Eqs. 3, 10, 11): work items visit the
-// texels in screen-space Hilbert order; texel t = (c, j) sits at distance
-// r = tan(e_c)/c_r from the gaze at angle phi = (j + 0.5) 360/n_c, so its
-// camera direction is (tan(e_c) cos(phi) + gx, -tan(e_c) sin(phi) + gy, 1).
-// Returns the texel's slot; `guard_lo` / `guard_hi` get the guard slots that
-// copy it (texel n_c - 1 -> slot before the column, texel 0 -> slot after),
-// or -1.
-__device__ __forceinline__ int lp_ray(const FrameDesc& f, int k, Ray& r, int& guard_lo, int& guard_hi) {
-    const int2 tc = __ldg(f.work + k);
+// LP ray of a work item, (slot, column) or number k of the frame's list (Eqs. 3,
+// 10, 11): work items visit the texels in screen-space Hilbert order; texel t =
+// (c, j) sits at distance r = tan(e_c)/c_r from the gaze at angle phi = (j + 0.5)
+// 360/n_c, so its camera direction is (tan(e_c) cos(phi) + gx, -tan(e_c) sin(phi) +
+// gy, 1).  Returns the texel's slot; `guard_lo` / `guard_hi` get the guard slots that
+// copy it (texel n_c - 1 -> slot before the column, texel 0 -> slot after), or -1.
+__device__ __forceinline__ int lp_ray(const FrameDesc& f, int2 tc, Ray& r, int& guard_lo, int& guard_hi) {
     const int2 cc = __ldg(&f.col[tc.y]);
     const int j = tc.x - cc.x;
     const float te = __ldg(&f.tan_e[tc.y]);
@@ -559,6 +557,9 @@ __device__ __forceinline__ int lp_ray(const FrameDesc& f, int k, Ray& r, int& gu
     guard_lo = j == cc.y - 1 ? tc.x - cc.y : -1;
     guard_hi = j == 0 ? tc.x + cc.y : -1;
     return tc.x;
+}
+__device__ __forceinline__ int lp_ray(const FrameDesc& f, int k, Ray& r, int& guard_lo, int& guard_hi) {
+    return lp_ray(f, __ldg(f.work + k), r, guard_lo, guard_hi);
 }
 
 // Shaded LP texel (and hit id) into its slot and the guard slots that copy it.

@@ -241,6 +241,11 @@ void count_launch(int k = 1);
 // reconstruction 35.3 -> 33.3 (back to back), a 1280 x 720 frame of 64 triangles 63.6
 // -> 60.4, with FXAA 89.5 -> 83.9, the warped 8K eye 370 -> 362.  (Casts that let the
 // next launch in at their start instead of at their end gain nothing more.)
+// Such a kernel has begun while the one before it may still write, so memory that
+// an earlier launch writes is not constant for the kernel's whole life, as __ldg and
+// ld.global.nc require: buffers of the frame (LP texels, lumas, depths, lists of
+// work, visibility) are read by plain loads, which stay behind the wait.  __ldg is
+// for the scene and for the layout's tables, which no overlapped launch writes.
 __device__ __forceinline__ void after_previous() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
