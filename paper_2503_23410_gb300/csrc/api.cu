@@ -2,8 +2,11 @@
 // lifetimes, argument checking, the FP64 host set-up of the log-polar layout
 // (Sec. 3.2.2, Eqs. 9, 10, 12) and of each frame's gaze parameters (Eq. 3),
 // batching, CUDA-graph capture and the tile-shape autotuner.
+#include "inputs.h"
 #include "layout.h"
 #include "vafr_internal.cuh"
+
+#include <cuda.h>
 
 #include <algorithm>
 #include <atomic>
@@ -103,6 +106,44 @@ bool is_device_ptr(const void* p) {
         return false;
     }
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
+}
+
+// The allocation that holds device address p, as the driver knows it; size 0 if it
+// knows none.  (The call is found through the runtime, so the library needs no
+// link against the driver.)
+void allocation_of(const void* p, uintptr_t* base, size_t* size) {
+    using GetRange = CUresult (*)(CUdeviceptr*, size_t*, CUdeviceptr);
+    static std::atomic<GetRange> found{nullptr};
+    GetRange get = found.load();
+    if (!get) {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &q) != cudaSuccess)
+            cudaGetLastError();
+        else if (q == cudaDriverEntryPointSuccess)
+            found = get = reinterpret_cast<GetRange>(f);
+    }
+    CUdeviceptr b = 0;
+    *base = 0;
+    *size = 0;
+    if (get && get(&b, size, reinterpret_cast<CUdeviceptr>(p)) == CUDA_SUCCESS)
+        *base = (uintptr_t)b;
+    else
+        *size = 0;
+}
+
+// Whether a build on `device` reads `bytes` bytes of floats at device pointer p in place.
+bool reads_in_place(const void* p, size_t bytes, int device) {
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    uintptr_t base = 0;
+    size_t size = 0;
+    allocation_of(p, &base, &size);
+    const bool here = a.type == cudaMemoryTypeManaged || (a.type == cudaMemoryTypeDevice && a.device == device);
+    return readable_in_place(here, reinterpret_cast<uintptr_t>(p), bytes, base, size);
 }
 
 int bytes_per_px(int fmt) { return fmt == VAFR_FMT_RGBA16F ? 8 : 16; }
@@ -500,8 +541,7 @@ static int vafr_build_scene_impl(const float* tri_xyz, const float* albedo_rgb, 
     if (cudaMemsetAsync(sc->status, 0, sizeof(unsigned), s) != cudaSuccess)
         return bail(fail(VAFR_ERR_CUDA, "memset status"));
     if (n > 0) {
-        // device inputs are read where they are, host inputs and those between two
-        // floats' addresses copied first
+        // device inputs are read where they are if they can be (inputs.h), all others copied first
         struct Copy {   // freed on every way out
             float* p = nullptr;
             ~Copy() { if (p) cudaFree(p); }
@@ -509,8 +549,8 @@ static int vafr_build_scene_impl(const float* tri_xyz, const float* albedo_rgb, 
         b.tris = tri_xyz;
         b.albedo = albedo_rgb;
         auto to_device = [&](Copy& c, const float** in, size_t count) -> cudaError_t {
-            const bool device = *in && is_device_ptr(*in);
-            if (!*in || (device && aligned(*in, sizeof(float)))) return cudaSuccess;
+            if (!*in || reads_in_place(*in, sizeof(float) * count, sc->device)) return cudaSuccess;
+            const bool device = is_device_ptr(*in);
             cudaError_t e = cudaMalloc(&c.p, sizeof(float) * count);
             if (e == cudaSuccess)
                 e = cudaMemcpyAsync(c.p, *in, sizeof(float) * count,
