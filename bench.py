@@ -70,9 +70,20 @@ PT_DIFFUSE = 3        # the paper's maximum diffuse bounces (Sec. 8.1)
 # is the pixel ray (15), the shear set-up (3 abs, 5 compares/selects, 2 divides
 # + 1 reciprocal, 9 selects = 20), the watertight test on eye-relative
 # vertices (50) and the key (3).
-LPT_VARIANTS = (0, 6, 7)   # render variants in longest-first chunk order (k_render_lp_lpt)
+PLAIN_TRIS = 4096          # render variant 0 casts scenes up to this size in plain order
+LPT_VARIANTS = (6, 7)      # render variants in longest-first chunk order (k_render_lp_lpt) in every scene
 OPS_PER_PREFILTER = 13
 OPS_PER_PIXEL_TEST = 88
+
+
+def longest_first(variant, n_tris):
+    """Whether a session's LP casts of n_tris triangles run k_render_lp_lpt."""
+    return variant in LPT_VARIANTS or (variant == 0 and n_tris > PLAIN_TRIS)
+
+
+def gt_variants(n_variants):
+    """Render variants that differ in the full-resolution cast: variants 6 and 7 are variant 4 there."""
+    return [v for v in range(n_variants) if v not in LPT_VARIANTS]
 
 
 def _dist():
@@ -387,13 +398,11 @@ def run_gpu(args, w):
             V.vafr_session_tuning(sess, vafr_cfg)
 
     if not (pt or deferred):
-        # pick it: every plain-order render variant casts one untimed and two
+        # pick it: every render variant with a kernel of its own casts one untimed and two
         # timed GT frames (CUDA events), the fastest is kept
         vafr_cfg = V.vafr_session_tuning(sess)
         best = None
-        for v in range(V.vafr_tuning_space()[0]):
-            if v in LPT_VARIANTS:
-                continue
+        for v in gt_variants(V.vafr_tuning_space()[0]):
             V.vafr_session_tuning(sess, (v, vafr_cfg[1]))
             for e in range(eyes):
                 V.vafr_render_full_gt(scene, sess, e, disp[e * dp_b:])
@@ -562,7 +571,7 @@ def run_gpu(args, w):
     # traffic lines were captured with the paper's acuity model; another model
     # changes the ray count and the LP buffer, so it needs captures of its own
     traffic_key = args.workload if args.acuity == "paper" else f"{args.workload}+{args.acuity}"
-    lpt = bool(tuning) and tuning[0] in LPT_VARIANTS
+    lpt = bool(tuning) and longest_first(tuning[0], w.scene.n_tris)
     if pt:
         tr_render, _ = _traffic("path_lp", [os.path.join(csrc, f) for f in ("pathtrace.cu", "trace.cuh")],
                                 traffic_key)
