@@ -321,18 +321,10 @@ cudaError_t lpt_next(LptState* st, unsigned& frames, cudaStream_t s, LptState** 
     return cudaSuccess;
 }
 
-// Scratch of a pooled path tracing launch: the session's; NULL, for the kernel that
-// needs none, for little work and until path_scratch_next has allocated it.
-void* path_scratch(const vafr_session* s, long long work, int depth) {
-    return path_uses_pool(work, depth) ? s->d_path : nullptr;
-}
-
-// After a launch that could have used the scratch: allocates it for the next one
-// while the GPU works (10 MB, some 170 us: before the first launch it made a
-// 490 us path tracing pass 530).  A failure leaves the session without.  The relaxed
-// mode keeps it from ending a capture that is under way, on this call's stream or
-// another thread's.
-void path_scratch_next(vafr_session* s, long long work, int depth) {
+// Path tracing's scratch for later launches of the session (10 MB).  A failure leaves
+// the session without.  The relaxed mode keeps the allocation from ending a capture
+// that is under way, on this call's stream or another thread's.
+void path_scratch_alloc(vafr_session* s, long long work, int depth) {
     if (s->d_path || !path_uses_pool(work, depth)) return;
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
     if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) {
@@ -344,6 +336,19 @@ void path_scratch_next(vafr_session* s, long long work, int depth) {
         s->d_path = nullptr;
     }
     cudaThreadExchangeStreamCaptureMode(&mode);
+}
+
+// Scratch of a pooled path tracing launch: the session's; NULL, for the kernel that
+// needs none, for little work and for a session's first launch, behind which the
+// caller allocates it while the GPU works (some 170 us: before the first launch it
+// made a 490 us path tracing pass 530).  A captured launch lasts as long as its
+// graph and nothing waits for it yet: its scratch is allocated first.
+void* path_scratch(vafr_session* s, long long work, int depth, cudaStream_t st) {
+    if (!path_uses_pool(work, depth)) return nullptr;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (!s->d_path && cudaStreamIsCapturing(st, &capture) != cudaSuccess) cudaGetLastError();
+    if (capture != cudaStreamCaptureStatusNone) path_scratch_alloc(s, work, depth);
+    return s->d_path;
 }
 
 int lpt_chunks(int64_t n_texels) { return (int)((n_texels + kLptChunk - 1) / kLptChunk); }
@@ -909,9 +914,9 @@ int vafr_render_lp_pt(const vafr_scene* scene, vafr_session* s, int32_t eye_mask
         b.total_work += s->n_texels;
         b.d[b.n++] = f;
     }
-    void* scratch = path_scratch(s, b.total_work, max_diffuse);
+    void* scratch = path_scratch(s, b.total_work, max_diffuse, as_stream(stream));
     CUDA_TRY(launch_path_lp(scene->dev, b, (unsigned long long)seed, max_diffuse, scratch, as_stream(stream), s->sms));
-    path_scratch_next(s, b.total_work, max_diffuse);
+    path_scratch_alloc(s, b.total_work, max_diffuse);
     return VAFR_OK;
 }
 
@@ -1149,9 +1154,9 @@ int vafr_render_full_gt_pt(const vafr_scene* scene, vafr_session* s, int32_t eye
     b.d[0] = f;
     b.n = 1;
     b.total_work = gt_items(f);
-    void* scratch = path_scratch(s, b.total_work, max_diffuse);
+    void* scratch = path_scratch(s, b.total_work, max_diffuse, as_stream(stream));
     CUDA_TRY(launch_path_gt(scene->dev, b, (unsigned long long)seed, max_diffuse, scratch, as_stream(stream), s->sms));
-    path_scratch_next(s, b.total_work, max_diffuse);
+    path_scratch_alloc(s, b.total_work, max_diffuse);
     return VAFR_OK;
 }
 
