@@ -42,7 +42,7 @@ def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
     os.makedirs(OBJ, exist_ok=True)
     headers = [os.path.join(CSRC, "vafr_internal.cuh"), os.path.join(CSRC, "layout.h"),
                os.path.join(CSRC, "lp_map.cuh"), os.path.join(CSRC, "trace.cuh"), os.path.join(CSRC, "inputs.h"),
-               os.path.join(HERE, "..", "include", "vafr.h")]
+               os.path.join(CSRC, "mesh_rule.h"), os.path.join(HERE, "..", "include", "vafr.h")]
     jobs = []
     for src in SOURCES:
         s = os.path.join(CSRC, src)

@@ -28,6 +28,7 @@
 //             uncovered ones are listed as holes and ray cast.
 // All arithmetic FP32 (the oracle does the same steps in FP64).
 #include "lp_map.cuh"
+#include "mesh_rule.h"
 #include "vafr_internal.cuh"
 
 namespace vafr {
@@ -129,27 +130,14 @@ __global__ void __launch_bounds__(256) k_rep_vertices(const __grid_constant__ Sm
 }
 
 // The compact indices of the three left texels of triangle s of left texel (c, j),
-// and the column of the third (see the mesh rule).  Rings below 32,768 texels keep
-// the products within 32 bits, and k, at most 3/2 ring sizes, needs one correction
-// and no remainder (the raster pass takes 38 us, with 64-bit divisions and
-// remainders 42).
+// and the column of the third (see the mesh rule).
 __device__ __forceinline__ bool rep_triangle(const int2* colt, int C, int c, int j, int s, int tv[3], int& c2) {
     c2 = s == 0 ? c + 1 : c - 1;
     if (c2 < 0 || c2 >= C) return false;
     const int2 a = __ldg(colt + c), b = __ldg(colt + c2);
-    long long k;
-    if ((a.y | b.y) < 32768) {
-        const unsigned n = (unsigned)a.y, num = (2u * (unsigned)j + 3u) * (unsigned)b.y;
-        k = s == 0 ? ((int)((num + n - 1u) / n) - 2) >> 1 : ((int)(num / n) - 1) >> 1;
-    } else {
-        const long long n = a.y, num = (2ll * j + 3) * b.y;
-        k = s == 0 ? ((num + n - 1) / n - 2) >> 1 : (num / n - 1) >> 1;
-    }
-    if (k < 0) k += b.y;
-    else if (k >= b.y) k -= b.y;
     tv[0] = a.x - guards(c) + j;
     tv[1] = a.x - guards(c) + (j + 1 == a.y ? 0 : j + 1);
-    tv[2] = b.x - guards(c2) + (int)k;
+    tv[2] = b.x - guards(c2) + ring_partner(a.y, b.y, j, s);
     return true;
 }
 
