@@ -270,11 +270,13 @@ VAFR_API int vafr_session_sizes(const vafr_session* session, int64_t* lp_bytes_p
                        int64_t* display_bytes_per_eye);
 /* Reads (set = 0) or writes (set = 1) the kernel variants used by this
  * session's single-session calls: cfg[0] render variant, cfg[1] reconstruct
- * tile shape (see vafr_tuning_space).  Render variants 6 and 7, and the
- * default 0 in scenes above 4,096 triangles, take the LP work in chunks of 32 rays and render the chunks that
- * were slowest in the session's previous frame first, so a launch does not end
- * waiting for slow chunks that happened to come last (7 keeps fewer registers,
- * 7 blocks per SM).  Results do not depend on the choice.
+ * tile shape (see vafr_tuning_space).  Render variants 6 and 7, and the default 0
+ * in scenes above 4,096 triangles, take the LP work in chunks of 32 rays and
+ * render the chunks that were slowest in the session's previous frame first, so a
+ * launch does not end waiting for slow chunks that happened to come last (7 keeps
+ * fewer registers, 7 blocks per SM).  Variant 5 visits only the nearest child
+ * first, which is faster in some scenes of large overlapping triangles.  Results do
+ * not depend on the choice.
  * Errors: INVALID_ARG (NULL, variant out of range). */
 VAFR_API int vafr_session_tuning(vafr_session* session, int32_t set, int32_t cfg[2]);
 /* Picks the session's kernel variants by timing whole frames at the current

@@ -886,7 +886,8 @@ int vafr_render_lp(const vafr_scene* scene, vafr_session* s, int32_t eye_mask, v
         f.hit_ids = hit_ids_out ? hit_ids_out + (size_t)b.n * s->n_slots : nullptr;
         f.work_begin = b.total_work;
         if (has_lpt_kernel(s->render_variant, scene->dev.n_tris))
-            CUDA_TRY(lpt_next(s->d_lpt[eye], s->lpt_frames[eye], as_stream(stream), &f.lpt, b.n ? nullptr : &b.work_counter));
+            CUDA_TRY(lpt_next(s->d_lpt[eye], s->lpt_frames[eye], as_stream(stream), &f.lpt,
+                              b.n ? nullptr : &b.work_counter));
         b.total_work += s->n_texels;
         b.d[b.n++] = f;
     }
@@ -981,7 +982,8 @@ int vafr_render_lp_rep(const vafr_scene* scene, vafr_session* s, void* lp_out, i
     b.d[0].work_begin = 0;
     b.n = 1;
     b.total_work = s->n_texels;
-    if (has_lpt_kernel(s->render_variant, scene->dev.n_tris)) CUDA_TRY(lpt_next(s->d_lpt[0], s->lpt_frames[0], st, &b.d[0].lpt, &b.work_counter));
+    if (has_lpt_kernel(s->render_variant, scene->dev.n_tris))
+        CUDA_TRY(lpt_next(s->d_lpt[0], s->lpt_frames[0], st, &b.d[0].lpt, &b.work_counter));
     CUDA_TRY(launch_render_lp(scene->dev, b, s->render_variant, st, s->sms));
     // 2. warp into the right eye
     SmallBatch w{};

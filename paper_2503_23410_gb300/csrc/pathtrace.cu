@@ -63,15 +63,17 @@ __device__ __forceinline__ float3 face_normal(const SceneDev& sc, const Ray& r, 
 // One path per lane from its first to its last segment leaves most lanes idle:
 // on the 1.07 M triangle terrain 93 % of the paths have a second segment but
 // 25 % a third and 16 % a fourth, and 14 %, 12 % and 7 % a shadow ray there,
-// while each of these steps takes a warp nearly as long as the full ones (308,
-// 695, 1,077 and 1,391 us for the LP buffer at 0 to 3 bounces, 10.6 of 32 lanes
-// active).  With the pool 1,391 us become 1,048 (15 lanes; the incoherent bounce
+// while each of these steps takes a warp nearly as long as the full ones (276,
+// 629, 974 and 1,252 us for the LP buffer at 0 to 3 bounces, 10.6 of 32 lanes
+// active).  With the pool 1,252 us become 945 (15 lanes; the incoherent bounce
 // rays' leaf tests and pushes are what diverges now).
 // The records also hold what the traversal does not need, so it fits 64
-// registers and kPathBlocks blocks per SM (one path per lane: 93 and 5; 6, 7
-// and 8 blocks measured 1,156, 1,148 and 1,110 us, and 1,064 with all four
-// children sorted).  What a ray does not need lies in global memory instead
-// of beside it in shared memory, where it took L1 from the nodes (1,172 us).
+// registers and kPathBlocks blocks per SM (one path per lane: 93 and 5).  When
+// the pool was made, on a traversal of more instructions that took 1,391 us with one
+// path per lane, 6, 7 and 8 blocks measured 1,156, 1,148 and 1,110 us, and 1,064
+// with all four children sorted.  What a ray does not need lies in global memory
+// instead of beside it in shared memory, where it took L1 from the nodes (1,172
+// us then).
 constexpr int kPathBlocks = 8;   // resident blocks per SM that the launch and its scratch count on
 constexpr int kPoolPaths = 64;   // fewer than 32 waiting, and the next 32
 struct PathPool {

@@ -190,13 +190,14 @@ __device__ __forceinline__ void flush_counts(const RasterCounts& n, unsigned lon
 // boxes, or of the tiles left of them, in turn: pre-filter, depth pre-test, and
 // what passes both goes into a queue that is tested exactly 32 pixels at a time.
 // Of the 88 M box pixels of a 4K frame of the 1.07 M triangle terrain 35 M pass
-// the pre-filter and 17 M the depth pre-test.  When each warp step ran the exact
-// test (some 150 instructions) for whichever lanes had passed, and a thread
-// rasterised its own small triangle (13 of 32 lanes busy), the visibility buffer
-// took 795 us; it took 465 so, and takes 411 since the triangle test shears by axis
-// (1080p 330 -> 241, 8K of 2 M triangles 5,430 -> 1,840).  kSteps depths are loaded before any is looked at, and the tile pass
-// hands out its work as it goes: with one load at a time and equal runs of tiles
-// it took 724 us.
+// the pre-filter and 20 M the depth pre-test (18 M where each is looked at only when
+// its turn to be tested has come).  When each warp step ran the exact test (some 150
+// instructions) for whichever lanes had passed, and a thread rasterised its own
+// small triangle (13 of 32 lanes busy), the visibility buffer took 800 us; it took
+// 465 so, and takes 411 since the triangle test shears by axis (1080p 331 -> 239, 8K
+// of 2 M triangles 5,430 -> 1,800).  kSteps depths are loaded before any is looked
+// at, and the tile pass hands out its work as it goes: with one load at a time and
+// equal runs of tiles it took 724 us before that.
 constexpr int kSteps = 4;   // pixels that a lane looks at before any is tested
 struct RasterWarp {
     float4 e[3][32];          // edge functions (ea, eb, ec, slack): inside where ea x + eb y + ec > -slack
@@ -312,7 +313,8 @@ k_vbuf_raster(const SceneDev sc, const __grid_constant__ SmallBatch b, unsigned 
     const unsigned lt = (1u << lane) - 1u;
     RasterCounts n{};
     const int n_warps = (int)gridDim.x * kRasterWarps;
-    for (int g = (int)blockIdx.x * kRasterWarps + (int)(threadIdx.x >> 5); (long long)g * per < sc.n_tris; g += n_warps) {
+    for (int g = (int)blockIdx.x * kRasterWarps + (int)(threadIdx.x >> 5); (long long)g * per < sc.n_tris;
+         g += n_warps) {
         const long long k = lane < per ? (long long)g * per + lane : sc.n_tris;
         int area = 0;
         int4 box = make_int4(0, 0, 0, 0);
@@ -619,8 +621,8 @@ cudaError_t launch_vbuffer(const SceneDev& sc, const SmallBatch& b, const VbufSc
                                                    per, nullptr);
     count_launch(1);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    return launch_overlapped(stats ? k_vbuf_tiles<true> : k_vbuf_tiles<false>, (unsigned)blocks, tpb, 0, s, sc, b, v.vbuf,
-                             v.big, v.big_leaf, v.big_first, v.counter, v.big_cap, stats);
+    return launch_overlapped(stats ? k_vbuf_tiles<true> : k_vbuf_tiles<false>, (unsigned)blocks, tpb, 0, s, sc, b,
+                             v.vbuf, v.big, v.big_leaf, v.big_first, v.counter, v.big_cap, stats);
 }
 
 cudaError_t launch_leaf_of(const SceneDev& sc, int* leaf_of, cudaStream_t s, int num_sms) {
@@ -634,11 +636,11 @@ cudaError_t launch_shade_vbuf(const SceneDev& sc, const SmallBatch& b, const uns
                               const int* leaf_of, bool full_res, cudaStream_t s, int num_sms) {
     if (full_res) {
         const long long n = (long long)b.d[0].W * b.d[0].H;
-        return launch_overlapped(k_shade_gt_vbuf, (unsigned)min((n + 255) / 256, (long long)num_sms * 16), 256, 0, s, sc, b,
-                                 vbuf, leaf_of);
+        return launch_overlapped(k_shade_gt_vbuf, (unsigned)min((n + 255) / 256, (long long)num_sms * 16), 256, 0, s,
+                                 sc, b, vbuf, leaf_of);
     }
-    return launch_overlapped(k_shade_lp_vbuf, (unsigned)min((b.d[0].n_texels + 255) / 256, num_sms * 16), 256, 0, s, sc, b,
-                             vbuf, leaf_of);
+    return launch_overlapped(k_shade_lp_vbuf, (unsigned)min((b.d[0].n_texels + 255) / 256, num_sms * 16), 256, 0, s,
+                             sc, b, vbuf, leaf_of);
 }
 
 }  // namespace vafr

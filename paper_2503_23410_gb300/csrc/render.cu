@@ -48,8 +48,9 @@ k_render_lp(const SceneDev sc, const __grid_constant__ B b) {
 // few (1-4 % of the texels), so with 32 rays to a warp most of the chip has
 // nothing to do and the launch lasts as long as its slowest warp, whose 32
 // rays at silhouettes go different ways.  Each warp instead takes as few rays
-// as still gives every resident warp some: at 30 K holes 7 rays a warp, and
-// the 8K binocular VaFR_Rep cast 488 -> 453 us (8 rays 463, 16 rays 474).
+// as still gives every resident warp some: with 10.5 K holes (1 %) the whole 8K
+// binocular VaFR_Rep call takes 362 us, 381 with 32 rays to a warp, 371 with 16 and
+// 365 with 8.
 __global__ void __launch_bounds__(128)
 k_render_list(const SceneDev sc, const __grid_constant__ SmallBatch b, const unsigned* count) {
     after_previous();

@@ -143,7 +143,8 @@ __device__ __forceinline__ unsigned key_limit(float t) {
 // the limit (a key_limit); key: the children's sort keys (child_key), all ones for
 // a miss.
 template <bool LIM>
-__device__ __forceinline__ void slab4(const float4* __restrict__ nd, const Ray& r, const uint4& word, unsigned lim, unsigned key[4]) {
+__device__ __forceinline__ void slab4(const float4* __restrict__ nd, const Ray& r, const uint4& word, unsigned lim,
+                                      unsigned key[4]) {
     float4 nxp, fxp, nyp, fyp, nzp, fzp;
     ldg256(nd + r.nx, nxp, fxp);
     ldg256(nd + r.ny, nyp, fyp);

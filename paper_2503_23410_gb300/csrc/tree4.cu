@@ -751,8 +751,8 @@ cudaError_t tree4_pack(const LbvhBuffers& b, void* scratch, int n_nodes4, cudaSt
     const int n = b.n;
     if (n <= 1) return cudaSuccess;
     const Tree4Scratch sc = carve(scratch, n);
-    k_pack_nodes4<<<blocks_for(4ll * n_nodes4, kThreads), kThreads, 0, s>>>(sc.nodes, b.leaf_box, sc.off, sc.sums, sc.head_of,
-                                                                      n - 1, n_nodes4, b.nodes4);
+    k_pack_nodes4<<<blocks_for(4ll * n_nodes4, kThreads), kThreads, 0, s>>>(sc.nodes, b.leaf_box, sc.off, sc.sums,
+                                                                            sc.head_of, n - 1, n_nodes4, b.nodes4);
     count_launch(1);
     return cudaGetLastError();
 }

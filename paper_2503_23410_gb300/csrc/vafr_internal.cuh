@@ -153,6 +153,24 @@ constexpr int kLptVariantLean = 7;
 // pays: the longest-first bookkeeping costs casts of 60 to 90 us 4 to 6 us, and
 // sorting changes soups of 500 to 4,000 triangles by -15 to +13 % from scene to
 // scene.
+// What decides is the scene, not its size; the line lies where the two about even
+// out.  At 1024 x 768, us, nearest child first | longest-first (casts) and sorted (GT),
+// for two or three scenes of each kind:
+//                         casts                                      GT
+//   terrain      700      83 74 | 84 75                              49 42 | 49 43
+//   triangles  2,700      101 85 | 94 84                             59 54 | 61 53
+//              7,000      103 94 | 87 87                             70 62 | 69 66
+//             1.07 M      176 173 | 151 144                          128 103 | 104 100
+//   soups of   1,000      394 623 | 405 642                          268 254 | 306 261
+//   triangles  4,000      1678 3312 | 1406 3273                      1068 1160 | 1010 1237
+//   as large  10,000      4551 8589 2038 | 4181 8544 2272            2774 2661 2070 | 2736 2744 2275
+//   as the    40,000      14084 21347 9496 | 15401 21275 10478       8050 6348 9267 | 9522 6813 9925
+//   scene     80,000      29489 58937 16602 | 24918 50180 17952      16656 16049 16186 | 15344 13960 17322
+//   a fifth  100,000      638 862 288 | 511 396 263                  576 695 318 | 552 288 316
+// The leaves' overlap does not separate them either: either order may win where the
+// boxes' areas add up to 50 or to 10,000 times the scene's.  A session's own choice is
+// vafr_session_autotune's; variant 5 puts the nearest child first in scenes of any
+// size, within 4 % of the 72-register kernel.
 constexpr int kPlainTris = 4096;
 // variants that render with a longest-first order in every batch ...
 __host__ __device__ constexpr bool is_lpt_variant(int v) { return v == kLptVariant || v == kLptVariantLean; }
