@@ -227,11 +227,12 @@ __device__ __forceinline__ int find_aa_frame(const B& b, long long w) {
 // one column (blockIdx.x; frame blockIdx.z), kLumaItems to a thread and all of them
 // loaded before the first is stored; the guard slots get the lumas of the texels
 // that they stand for, whatever the buffer's own guards hold.  It reads 17 MB and
-// writes 4 for an eye in FP32, so what counts is loads in flight: both passes take
-// 31.8 us with 128 threads of 8 rows, 32.1 with 256 of 4, 32.7 with 128 of 4, 35.5 with
-// 256 of one, all on one buffer; 33.5 over buffers in turn, where a pass over the
-// slots in order, which cannot tell a guard from a texel, took 33.2.
-constexpr int kLumaThreads = 128, kLumaItems = 8, kLumaParts = 2;
+// writes 4 for an eye in FP32, so what counts is loads in flight and blocks of about
+// the same length (rings have up to some 1,640 rows): both passes take 33.9 us over
+// buffers in turn with 128 threads of 7 rows, 34.4 with 8, 34.7 with 6 or 5, 34.0 with
+// 256 threads of 7, 34.4 of 3, 35.3 with 64 of 7; a pass over the slots in order,
+// which cannot tell a guard from a texel, 33.9.
+constexpr int kLumaThreads = 128, kLumaItems = 7, kLumaParts = 2;
 
 template <class B>
 __global__ void __launch_bounds__(kLumaThreads) k_lp_luma(const __grid_constant__ B b) {

@@ -421,9 +421,10 @@ __device__ __forceinline__ void ld_if(bool p, const int4* ptr, int4& v) {
 }
 
 // LP texel `idx` into `v` if `p`: FP32 RGBA, or FP16 RGBA widened exactly.  A plain
-// load, as the launch before may have written the texels (predicated inline
-// assembly, ordinary or volatile, takes the same 33.0 us for a 4K FP32 eye; through
-// the read-only path it took 32.7).
+// load, as the launch before may have written the texels; such loads do not pass the
+// stores of the rows before (through the read-only path a 4K FP32 eye took 32.6 us for
+// 32.9; predicated inline assembly takes 32.9 too; storing a pixel behind the next
+// row's loads 32.75, but its registers cost an 8K FP16 eye 116 -> 117).
 template <int LPF>
 __device__ __forceinline__ void ld_texel_if(bool p, const void* lp, int idx, px2& v) {
     if (p) v = load_lp(lp, LPF, idx);
