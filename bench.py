@@ -571,7 +571,7 @@ def run_gpu(args, w):
     # traffic lines were captured with the paper's acuity model; another model
     # changes the ray count and the LP buffer, so it needs captures of its own
     traffic_key = args.workload if args.acuity == "paper" else f"{args.workload}+{args.acuity}"
-    lpt = bool(tuning) and longest_first(tuning[0], w.scene.n_tris)
+    lpt = longest_first(tuning[0] if tuning else 0, w.scene.n_tris)   # untuned sessions have variant 0
     if pt:
         tr_render, _ = _traffic("path_lp", [os.path.join(csrc, f) for f in ("pathtrace.cu", "trace.cuh")],
                                 traffic_key)
@@ -583,7 +583,7 @@ def run_gpu(args, w):
     tr_recon, _ = _traffic("reconstruct", [os.path.join(csrc, f) for f in ("reconstruct.cu", "lp_map.cuh")],
                            traffic_key)
     render_kernel = ("k_path" if pt else
-                     "k_render_lp (left eye) + k_rep_* warp + k_render_list (holes)" if rep else
+                     f"k_render_lp{'_lpt' if lpt else ''} (left eye) + k_rep_* warp + k_render_list (holes)" if rep else
                      "k_render_lp_lpt" if lpt else "k_render_lp")
     roof_render = {"kernel": render_kernel, "bound": "alu",
                    "achieved": ops / render_s / 1e12,
