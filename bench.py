@@ -654,7 +654,7 @@ def run_gpu(args, w):
                "steps": gt_steps,
                "render_variant": (gt_variant if gt_variant is not None else
                                   V.vafr_session_tuning(sess)[0]),
-               "variant_by": ("fastest plain-order variant on 2 GT frames, picked before warm-up"
+               "variant_by": ("fastest variant on 2 GT frames, picked before warm-up"
                               if gt_variant is not None else "the VaFR frames' variant")},
         "speedup_vs_gt": gt_mean / float(step_ms.mean()),
         "stage_ms": dict({"render_lp": float(render_ms.mean()), "reconstruct": float(recon_ms.mean())},
