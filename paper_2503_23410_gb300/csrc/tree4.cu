@@ -699,7 +699,10 @@ cudaError_t tree4_build(const LbvhBuffers& b, void* scratch, cudaStream_t s, int
     // the attribute is the current device's and context's: every build sets it
     const cudaError_t big = cudaFuncSetAttribute(k_ploc_tail, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                  (int)sizeof(TailShared));
-    if (big != cudaSuccess) return big;
+    if (big != cudaSuccess) {
+        cudaGetLastError();   // it is returned, not left for a later call
+        return big;
+    }
     k_ploc_start<<<1, 1, 0, s>>>(sc.state, n);
     count_launch(1);
     PlocState st{n, 0, 0, 0};
